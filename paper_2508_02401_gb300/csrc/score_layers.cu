@@ -437,21 +437,13 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
         // item's arrival on the unit's counter after a warp barrier.
         bool ok = true;
         for (int it = 0;; ++it) {
-            int gi = -1, good = 1;
-            if (lane == 0) good = wait_item<kItemRing>(item_full, items, it, &gi, abort, lim) ? 1 : 0;
-            gi = __shfl_sync(0xffffffffu, gi, 0);
-            if (__shfl_sync(0xffffffffu, good, 0) == 0) {
-                ok = false;
-                break;
-            }
-            if (gi < 0) break;
+            int gi = -1;
+            ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
+            if (!ok || gi < 0) break;
             const Item I = get_item(p, gi);
             const int buf = it & 1;
-            if (lane == 0) good = mbar_wait(&pub_full[buf], (it >> 1) & 1, abort, lim) ? 1 : 0;
-            if (__shfl_sync(0xffffffffu, good, 0) == 0) {
-                ok = false;
-                break;
-            }
+            ok = __all_sync(0xffffffffu, mbar_wait(&pub_full[buf], (it >> 1) & 1, abort, lim));
+            if (!ok) break;
             double* dst = p.sums + static_cast<size_t>(I.unit) * N;
 #pragma unroll
             for (int c = lane; c < N; c += 32) {
@@ -568,14 +560,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
         int b_it = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            int gi = -1, good = 1;
-            if (lane == 0) good = wait_item<kItemRing>(item_full, items, it, &gi, abort, lim) ? 1 : 0;
-            gi = __shfl_sync(0xffffffffu, gi, 0);
-            if (__shfl_sync(0xffffffffu, good, 0) == 0) {
-                ok = false;
-                break;
-            }
-            if (gi < 0) break;
+            int gi = -1;
+            ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
+            if (!ok || gi < 0) break;
             // pass 2 reads an item's ring entry last: once each of its warps has, the producer
             // may post another item there
             if (lane == 0) mbar_arrive(&item_free[it % kItemRing]);

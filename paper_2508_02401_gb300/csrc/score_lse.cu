@@ -577,16 +577,10 @@ __global__ void __launch_bounds__(kThreads, 1) score_lse_layers_kernel(const __g
         int use = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            int gi = -1, good = 1;
-            if (lane == 0) {
-                good = wait_item<kLseItemRing>(item_full, items, it, &gi, abort, lim) ? 1 : 0;
-                mbar_arrive(&item_free[it % kLseItemRing]);
-            }
-            gi = __shfl_sync(0xffffffffu, gi, 0);
-            if (__shfl_sync(0xffffffffu, good, 0) == 0) {
-                ok = false;
-                break;
-            }
+            int gi = -1;
+            ok = __all_sync(0xffffffffu, wait_item<kLseItemRing>(item_full, items, it, &gi, abort, lim));
+            if (lane == 0) mbar_arrive(&item_free[it % kLseItemRing]);
+            if (!ok) break;
             if (gi < 0) break;
             const Item I = get_item(p, gi);
             const int n = I.ntiles;

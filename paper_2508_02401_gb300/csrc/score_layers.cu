@@ -275,6 +275,10 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
             // it1: items taken (pass-1 cursor on the last one); it2: pass-2 cursor
             int it1 = 0, jt1 = 0, use1 = 0, it2 = 0, jt2 = 0, use2 = 0, have2 = -1;
             Item I1{}, I2{};
+            const CUtensorMap *km1 = nullptr, *km2 = nullptr;
+            int g1 = 0, g2 = 0, tok1 = 0, tok2 = 0, once1 = 0;  // once1: tiles of the item loaded evict-first
+            int s1 = 0, s2 = 0;
+            uint32_t ph1 = 1, ph2 = 1;
             bool have1 = false, ended = false, ok = true;
             long long t0 = clock64();
             uint32_t idle = 0;
@@ -295,23 +299,28 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                             load_q(I1, qb);
                             have1 = true;
                             jt1 = 0;
+                            km1 = &p.tmap_k[I1.layer];
+                            g1 = p.batch_group[I1.batch];
+                            tok1 = I1.start + I1.tile0 * kTileKeys;
+                            // In a long unit pass 2 re-reads an item's first tiles too late for L2
+                            // anyway: loading them evict-first leaves L2 to the rest.
+                            once1 = I1.len > kLongUnitKeys ? (I1.ntiles + 4) / 5 : 0;
                         }
                         did = true;
                     }
                 }
                 if (have1) {
-                    const int s = use1 % kP1Slots;
-                    if (mbar_test(&free1[s], ((use1 / kP1Slots) & 1) ^ 1)) {
-                        mbar_arrive_expect_tx(&full1[s], kTileBytes);
-                        uint8_t* dst = ring1 + s * kTileBytes;
-                        const int g = p.batch_group[I1.batch];
-                        const int tok = I1.start + (I1.tile0 + jt1) * kTileKeys;
-                        const CUtensorMap* km = &p.tmap_k[I1.layer];
-                        // In a long unit pass 2 re-reads an item's first tiles too late for L2
-                        // anyway: loading them evict-first leaves L2 to the rest.
-                        const uint64_t polx = (I1.len > kLongUnitKeys && jt1 * 5 < I1.ntiles) ? pol2 : pol1;
-                        tma_load_3d_hint(dst, km, &full1[s], 0, g, tok, polx);
-                        tma_load_3d_hint(dst + kHalfBytes, km, &full1[s], 64, g, tok, polx);
+                    if (mbar_test(&free1[s1], ph1)) {
+                        mbar_arrive_expect_tx(&full1[s1], kTileBytes);
+                        uint8_t* dst = ring1 + s1 * kTileBytes;
+                        const uint64_t polx = jt1 < once1 ? pol2 : pol1;
+                        tma_load_3d_hint(dst, km1, &full1[s1], 0, g1, tok1, polx);
+                        tma_load_3d_hint(dst + kHalfBytes, km1, &full1[s1], 64, g1, tok1, polx);
+                        tok1 += kTileKeys;
+                        if (++s1 == kP1Slots) {
+                            s1 = 0;
+                            ph1 ^= 1;
+                        }
                         ++use1;
                         did = true;
                         if (++jt1 == I1.ntiles) {
@@ -325,16 +334,20 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                     if (have2 != it2) {
                         I2 = get_item(p, items[it2 % kItemRing]);
                         have2 = it2;
+                        km2 = &p.tmap_k[I2.layer];
+                        g2 = p.batch_group[I2.batch];
+                        tok2 = I2.start + I2.tile0 * kTileKeys;
                     }
-                    const int s = use2 % kP2Slots;
-                    if (mbar_test(&free2[s], ((use2 / kP2Slots) & 1) ^ 1)) {
-                        mbar_arrive_expect_tx(&full2[s], kTileBytes);
-                        uint8_t* dst = ring2 + s * kTileBytes;
-                        const int g = p.batch_group[I2.batch];
-                        const int tok = I2.start + (I2.tile0 + jt2) * kTileKeys;
-                        const CUtensorMap* km = &p.tmap_k[I2.layer];
-                        tma_load_3d_hint(dst, km, &full2[s], 0, g, tok, pol2);
-                        tma_load_3d_hint(dst + kHalfBytes, km, &full2[s], 64, g, tok, pol2);
+                    if (mbar_test(&free2[s2], ph2)) {
+                        mbar_arrive_expect_tx(&full2[s2], kTileBytes);
+                        uint8_t* dst = ring2 + s2 * kTileBytes;
+                        tma_load_3d_hint(dst, km2, &full2[s2], 0, g2, tok2, pol2);
+                        tma_load_3d_hint(dst + kHalfBytes, km2, &full2[s2], 64, g2, tok2, pol2);
+                        tok2 += kTileKeys;
+                        if (++s2 == kP2Slots) {
+                            s2 = 0;
+                            ph2 ^= 1;
+                        }
                         ++use2;
                         did = true;
                         if (++jt2 == I2.ntiles) {
@@ -348,8 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                     idle = 0;
                     t0 = clock64();
                 } else {
-                    __nanosleep(32u << (idle < 1u ? idle : 1u));
-                    if ((++idle & 15u) == 0u && (*abort || clock64() - t0 > lim)) {
+                    if ((++idle & 63u) == 0u && (*abort || clock64() - t0 > lim)) {
                         ok = false;
                         break;
                     }
@@ -372,63 +384,69 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
     } else if (warp == 1 || warp == 2) {
         // ------------------------------------------------------------ MMA issuers
         // warp 1: pass 1, warp 2: pass 2, so that neither pass's issue waits behind the other's.
-        if (lane == 0) {
-            const bool first = warp == 1;
-            const int nslots = first ? kP1Slots : kP2Slots;
-            const uint8_t* ring = first ? ring1 : ring2;
-            uint64_t* full = first ? full1 : full2;
-            uint64_t* freed = first ? free1 : free2;
-            uint64_t* acc_full = first ? a_full : b_full;
-            uint64_t* acc_empty = first ? a_empty : b_empty;
-            uint64_t* fin = first ? done : done + 1;
-            const uint32_t d0 = tmem_base + static_cast<uint32_t>((first ? 0 : kAcc) * N);
-            int use = 0;
-            bool ok = true;
-            for (int it = 0; ok; ++it) {
-                int gi = -1;
-                if (!wait_item<kItemRing>(item_full, items, it, &gi, abort, lim)) {
-                    ok = false;
-                    break;
-                }
-                if (gi < 0) break;
-                const int n = get_item(p, gi).ntiles;
-                const int qb = it % kQBufs;
-                if (!mbar_wait(&q_full[qb], (it / kQBufs) & 1, abort, lim)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t b0 = smem_u32(qbuf + qb * SL::kQBytes);
-                for (int jt = 0; jt < n; ++jt, ++use) {
-                    const int s = use % nslots, acc = use % kAcc;
-                    if (!mbar_wait(&full[s], (use / nslots) & 1, abort, lim) ||
-                        !mbar_wait(&acc_empty[acc], ((use / kAcc) & 1) ^ 1, abort, lim)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    const uint32_t a0 = smem_u32(ring + s * kTileBytes);
-                    const uint32_t d = d0 + static_cast<uint32_t>(acc * N);
-#pragma unroll
-                    for (int kk = 0; kk < kHeadDim / 16; ++kk) {
-                        const uint32_t koff = (kk & 3) * 32;
-                        const uint64_t ad = sdesc_k_major_sw128(a0 + (kk >> 2) * kHalfBytes + koff);
-                        const uint64_t bd = sdesc_k_major_sw128(b0 + (kk >> 2) * SL::kQHalf + koff);
-                        umma_bf16(d, ad, bd, kIdesc, kk > 0 ? 1u : 0u);
-                    }
-                    umma_commit(&acc_full[acc]);
-                    umma_commit(&freed[s]);
-                }
+        // The whole warp runs the loop and waits, one elected lane issues: the descriptors then stay in
+        // uniform registers (a tile's eight MMAs issued in 155 cycles; from a lane-0 branch, 597).
+        const bool leader = elect_one();
+        const bool first = warp == 1;
+        const int nslots = first ? kP1Slots : kP2Slots;
+        const uint64_t ring_desc = sdesc_k_major_sw128(smem_u32(first ? ring1 : ring2));
+        const uint64_t q_desc = sdesc_k_major_sw128(smem_u32(qbuf));
+        uint64_t* full = first ? full1 : full2;
+        uint64_t* freed = first ? free1 : free2;
+        uint64_t* acc_full = first ? a_full : b_full;
+        uint64_t* acc_empty = first ? a_empty : b_empty;
+        uint64_t* fin = first ? done : done + 1;
+        const uint32_t d0 = tmem_base + static_cast<uint32_t>((first ? 0 : kAcc) * N);
+        int s = 0, acc = 0;
+        uint32_t sph = 0, aph = 1;
+        bool ok = true;
+        for (int it = 0; ok; ++it) {
+            int gi = -1;
+            ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
+            if (!ok || gi < 0) break;
+            const int n = get_item(p, gi).ntiles;
+            const int qb = it % kQBufs;
+            ok = __all_sync(0xffffffffu, mbar_wait(&q_full[qb], (it / kQBufs) & 1, abort, lim));
+            if (!ok) break;
+            const uint64_t bd = q_desc + static_cast<uint64_t>(qb * (SL::kQBytes >> 4));
+            for (int jt = 0; jt < n; ++jt) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[s], sph, abort, lim) &&
+                                                 mbar_wait(&acc_empty[acc], aph, abort, lim));
                 if (!ok) break;
-                umma_commit(&q_empty[qb]);  // this pass is done with the item's query rows
+                tc_fence_after_sync();
+                const uint64_t ad = ring_desc + static_cast<uint64_t>(s * (kTileBytes >> 4));
+                const uint32_t d = d0 + static_cast<uint32_t>(acc * N);
+                if (leader) {
+#pragma unroll
+                    for (int kk = 0; kk < kHeadDim / 16; ++kk)
+                        umma_bf16(d, ad + (((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4),
+                                  bd + (((kk >> 2) * SL::kQHalf + (kk & 3) * 32) >> 4), kIdesc, kk > 0 ? 1u : 0u);
+                    umma_commit(&freed[s]);
+                    umma_commit(&acc_full[acc]);
+                }
+                __syncwarp();
+                if (++s == nslots) {
+                    s = 0;
+                    sph ^= 1;
+                }
+                if (++acc == kAcc) {
+                    acc = 0;
+                    aph ^= 1;
+                }
             }
+            if (ok && leader) umma_commit(&q_empty[qb]);  // this pass is done with the item's query rows
+            __syncwarp();
+        }
+        if (leader) {
             if (!ok) {
                 *abort = 1;
                 record_error(p.status, kDevTimeout, first ? 11 : 12);
             }
             umma_commit(fin);
-            volatile int never = 0;
-            mbar_wait(fin, 0, &never);
         }
+        __syncwarp();
+        volatile int never = 0;
+        mbar_wait(fin, 0, &never);
         __syncwarp();
     } else if (warp == 3) {
         // ------------------------------------------------------------ publisher

@@ -16,12 +16,12 @@
 // a unit's items finish close together and pass 2 re-reads its tiles while they are still in
 // L2.  No wait can close a cycle: a CTA waits only for units it holds an item of, a unit's
 // items are taken before any later unit's, and a CTA takes an item only when it can run its
-// pass 1 (up to two items ahead of its pass 2); if a unit's items were all held by CTAs that
-// cannot start them, each would hold three of the unit's items, more than the G it has.
+// pass 1 (a query buffer is free: up to one item ahead of its pass 2), so that no item that has
+// been taken waits for pass 2 of another.
 //
-// Exchange: at the end of an item, pass 1 leaves, per window-row column, its keys' sum
-// sum_j 2^(x_j) (x = logit * log2 e) as (m, s) with the item's maximum m in shared memory; a
-// publisher warp adds each s * 2^m in fp64 to the unit's accumulator with one atomic add and
+// Exchange: at the end of an item, each pass-1 warp leaves, per window-row column, its keys' sum
+// sum_j 2^(x_j) (x = logit * log2 e) as (m, s) with its keys' maximum m in shared memory; a
+// publisher warp combines them and adds each s * 2^m in fp64 to the unit's accumulator with one atomic add and
 // counts the item's arrival on the unit's counter with a release (the wait for its adds to
 // land stays off pass 1's path).  A unit's lse per column is log2 of its accumulator once the
 // counter is complete: one read of N doubles, whatever the number of items.  fp64 holds
@@ -40,8 +40,8 @@
 //   warp 1       allocates TMEM and issues the pass-1 tcgen05.mma (M = 128 keys, N = the
 //                window rows of a head batch, K = 128) into four pass-1 accumulators;
 //   warp 2       issues the pass-2 tcgen05.mma into four pass-2 accumulators;
-//   warp 3       the publisher: per item, the fp64 atomic adds of its column sums and the
-//                release of its arrival on the unit's counter;
+//   warp 3       the publisher: per item, its column sums from the pass-1 warps', their fp64 atomic
+//                adds and the release of its arrival on the unit's counter;
 //   warps 4-11   pass 1, one warpgroup per 32 columns: each thread owns one key (one TMEM
 //                lane) and keeps a running (max, sum of 2^(x - max)) per column;
 //   warps 12-15  pass 2, one warpgroup over all N columns: per item, a bounded acquire spin
@@ -59,10 +59,14 @@ namespace ckv {
 
 namespace {
 
-constexpr int kP1Slots = 2;   // pass-1 ring (HBM)
+// Rings of 128-key tiles and query-row buffers share the block's shared memory.  32 layers, us a call
+// at L = 131072 / 32768 / the ragged batch, slots of pass 1, of pass 2 and query buffers:
+//   2 / 3 / 3: 2001 / 636 / 1168    3 / 3 / 2: 1941 / 614 / 1092    2 / 4 / 2: 2002 / 636 / 1162
+//   4 / 2 / 2: 2191 / 680 / 1228    3 / 2 / 3: 2612 / 810 / 1502
+constexpr int kP1Slots = 3;   // pass-1 ring (HBM)
 constexpr int kP2Slots = 3;   // pass-2 ring (L2): pass 2 must outrun pass 1 after each exchange wait
 constexpr int kAcc = 4;       // TMEM accumulators per pass
-constexpr int kQBufs = 3;     // query-row buffers: pass 1 runs up to two items ahead of pass 2
+constexpr int kQBufs = 2;     // query-row buffers: pass 1 runs up to one item ahead of pass 2
 // Units of more keys than this (16 MB of K, an eighth of L2) load the first fifth of each item's
 // tiles evict-first in pass 1: their re-reads come after most of L2 has turned over.
 constexpr int kLongUnitKeys = 65536;
@@ -78,58 +82,36 @@ struct LayersSmem {
     static constexpr int kQ = kP2 + kP2Slots * kTileBytes;
     static constexpr int kQBytes = N * 256;             // one item's rows: N x 128 bf16
     static constexpr int kQHalf = N * 128;              // 64 dims of them
-    static constexpr int kBars = kQ + kQBufs * kQBytes;
+    static constexpr int kSums = kQ + kQBufs * kQBytes;  // float2[4][N]: (max, sum) per pass-1 warp and column
+    static constexpr int kNlse = kSums + 4 * N * 8;      // float[N]: -lse per column of pass 2's item
+    static constexpr int kBars = kNlse + N * 4;
     // mbarrier indices, in this order
     static constexpr int kFull1 = 0, kFree1 = kFull1 + kP1Slots, kFull2 = kFree1 + kP1Slots,
                          kFree2 = kFull2 + kP2Slots, kAFull = kFree2 + kP2Slots,
                          kAEmpty = kAFull + kAcc, kBFull = kAEmpty + kAcc, kBEmpty = kBFull + kAcc,
                          kQFull = kBEmpty + kAcc, kQEmpty = kQFull + kQBufs,
-                         kDone = kQEmpty + kQBufs, kGroup = kDone + 2,  // A0 A1 B
-                         kPubFull = kGroup + 3, kPubEmpty = kPubFull + 2,
-                         kItemFull = kPubEmpty + 2, kItemFree = kItemFull + kItemRing,
+                         kDone = kQEmpty + kQBufs, kGroup = kDone + 2,  // pass 2
+                         kPubFull = kGroup + 1, kPubEmpty = kPubFull + 1,
+                         kItemFull = kPubEmpty + 1, kItemFree = kItemFull + kItemRing,
                          kNumBars = kItemFree + kItemRing;
     static constexpr int kItems = kBars + 8 * kNumBars;  // int[kItemRing]: posted item indices
     static constexpr int kTmemSlot = kItems + 4 * kItemRing;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
-    static constexpr int kDynamic = kBytes + 1024;      // slack to align the base to 1024 B
 };
-// dynamic + the kernel's static shared memory (under 6 KB) within the 227 KB a block may use
-static_assert(LayersSmem<64>::kDynamic + 6 * 1024 <= 232448, "shared memory, N = 64");
+// All of the block's shared memory is dynamic, so its base is 1024-aligned (checked by the kernel).
+static_assert(LayersSmem<64>::kBytes <= 232448, "shared memory, N = 64");
 
-// End of a pass-1 item for one warpgroup of kCols columns: per column, the warp maximum by
-// redux and the sums rescaled to it, the warps' sums by recursive halving, then the four warps
-// through shared memory `red`; thread c < kCols (the warpgroup's first warp) leaves column c's
-// (max, sum) in `out[c]` once the publisher is done with that buffer's previous item, and
-// arrives on pub_full.
-__device__ __forceinline__ bool item_sums(float (&m)[kCols], float (&s)[kCols], float2* red, int eq,
-                                          int lane, int wtid, uint64_t* gbar, uint32_t& gphase,
-                                          uint64_t* pub_full, uint64_t* pub_empty, uint32_t pub_phase,
-                                          float2* out, volatile int* abort, long long lim) {
+// End of a pass-1 item for one warp of 32 keys: per column, the warp maximum by redux and the sums
+// rescaled to it, then the lanes' sums by recursive halving: lane l holds column l's (m[0], s[0]).
+__device__ __forceinline__ void warp_sums(float (&m)[kCols], float (&s)[kCols], int lane) {
 #pragma unroll
     for (int i = 0; i < kCols; ++i) {
         const float M = redux_max(m[i]);
         s[i] *= ex2_approx(m[i] - M);
         m[i] = M;
     }
-    transpose_reduce<kCols>(s, m, lane);  // lane l: column l
-    red[eq * 32 + lane] = make_float2(m[0], s[0]);
-    if (!group_sync(gbar, gphase, abort, lim)) return false;
-    if (wtid < kCols) {
-        float M = red[wtid].x;
-#pragma unroll
-        for (int q = 1; q < 4; ++q) M = fmaxf(M, red[q * 32 + wtid].x);
-        float S = 0.f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 x = red[q * 32 + wtid];
-            S += x.y * ex2_approx(x.x - M);
-        }
-        if (!mbar_wait(pub_empty, pub_phase ^ 1, abort, lim)) return false;
-        out[wtid] = make_float2(M, S);
-        mbar_arrive(pub_full);
-    }
-    return true;
+    transpose_reduce<kCols>(s, m, lane);
 }
 
 // s * 2^M as a double, for |M| <= kMaxLog2: the power of two of floor(M) exactly (built from
@@ -150,9 +132,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
     using SL = LayersSmem<N>;
     constexpr uint32_t kIdesc = idesc_bf16_f32(kTileKeys, N);
 
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t* ring1 = sm + SL::kP1;
     uint8_t* ring2 = sm + SL::kP2;
     uint8_t* qbuf = sm + SL::kQ;
@@ -168,21 +148,23 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
     uint64_t* q_full = bars + SL::kQFull;
     uint64_t* q_empty = bars + SL::kQEmpty;
     uint64_t* done = bars + SL::kDone;
-    uint64_t* group = bars + SL::kGroup;        // one per epilogue warpgroup: A0 A1 B
-    uint64_t* pub_full = bars + SL::kPubFull;   // pass 1 left an item's sums in pub_s[item parity]
-    uint64_t* pub_empty = bars + SL::kPubEmpty; // the publisher is done with pub_s[item parity]
+    uint64_t* group = bars + SL::kGroup;        // the pass-2 warpgroup's barrier
+    uint64_t* pub_full = bars + SL::kPubFull;   // pass 1 left an item's sums in sums_s
+    uint64_t* pub_empty = bars + SL::kPubEmpty; // the publisher has read them
     uint64_t* item_full = bars + SL::kItemFull; // items[k] holds the CTA's next item index
     uint64_t* item_free = bars + SL::kItemFree; // every role has read items[k]
     int* items = reinterpret_cast<int*>(sm + SL::kItems);
-    // scratch of the epilogues (static, so that its accesses are shared-memory instructions)
-    __shared__ float2 red_a[2][2][128];  // [item parity][warpgroup][warp * 32 + lane]
-    __shared__ float2 pub_s[2][64];      // [item parity][column]: (max, sum) of an item
-    __shared__ __align__(16) float nlse_s[64];  // -lse per column of pass 2's item
+    float2* sums_s = reinterpret_cast<float2*>(sm + SL::kSums);
+    float* nlse_s = reinterpret_cast<float*>(sm + SL::kNlse);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + SL::kTmemSlot);
     volatile int* abort = reinterpret_cast<volatile int*>(sm + SL::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_items = p.n_items;
+    if ((smem_u32(sm) & 1023u) != 0) {  // the swizzled tiles need it; uniform over the grid
+        if (threadIdx.x == 0) record_error(p.status, kDevTimeout, 9);
+        return;
+    }
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kP1Slots; ++i) {
@@ -205,11 +187,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
         }
         mbar_init(&done[0], 1);
         mbar_init(&done[1], 1);
-        for (int i = 0; i < 3; ++i) mbar_init(&group[i], kGroupArrivals);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&pub_full[i], 32 * kNW);  // the columns' threads of each pass-1 warpgroup
-            mbar_init(&pub_empty[i], 1);
-        }
+        mbar_init(group, kGroupArrivals);
+        mbar_init(pub_full, 4 * kNW);  // the pass-1 warps
+        mbar_init(pub_empty, 1);
         for (int i = 0; i < kItemRing; ++i) {
             mbar_init(&item_full[i], 1);
             mbar_init(&item_free[i], 4);  // one arrival per pass-2 warp, once it has read the entry
@@ -459,25 +439,34 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
             ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
             if (!ok || gi < 0) break;
             const Item I = get_item(p, gi);
-            const int buf = it & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(&pub_full[buf], (it >> 1) & 1, abort, lim));
+            ok = __all_sync(0xffffffffu, mbar_wait(pub_full, it & 1, abort, lim));
             if (!ok) break;
             double* dst = p.sums + static_cast<size_t>(I.unit) * N;
+            float2 ms[N / 32];
 #pragma unroll
-            for (int c = lane; c < N; c += 32) {
-                const float2 ms = pub_s[buf][c];
-                if (ms.y > 0.f) {
-                    if (!(fabsf(ms.x) <= static_cast<float>(kMaxLog2))) record_error(p.status, kDevRange, c);
-                    else atomicAdd(dst + c, scaled_sum(ms.x, ms.y));
+            for (int i = 0; i < N / 32; ++i) {  // the four warps of the column's warpgroup
+                float2 x[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[q] = sums_s[q * N + lane + 32 * i];
+                ms[i].x = fmaxf(fmaxf(x[0].x, x[1].x), fmaxf(x[2].x, x[3].x));
+                ms[i].y = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) ms[i].y += x[q].y * ex2_approx(x[q].x - ms[i].x);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(pub_empty);
+#pragma unroll
+            for (int i = 0; i < N / 32; ++i) {
+                const int c = lane + 32 * i;
+                if (ms[i].y > 0.f) {
+                    if (!(fabsf(ms[i].x) <= static_cast<float>(kMaxLog2))) record_error(p.status, kDevRange, c);
+                    else atomicAdd(dst + c, scaled_sum(ms[i].x, ms[i].y));
                 }
             }
             // the warp barrier orders every lane's adds before lane 0's release, and a release
             // is cumulative: a thread that acquires the count sees the adds of every item counted
             __syncwarp();
-            if (lane == 0) {
-                red_release_add(p.counters + I.unit, 1);
-                mbar_arrive(&pub_empty[buf]);
-            }
+            if (lane == 0) red_release_add(p.counters + I.unit, 1);
         }
         if (!ok && lane == 0) {
             *abort = 1;
@@ -490,11 +479,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
         const int wg = (warp - kWarpA) >> 2;  // columns [wg*32, wg*32+32)
         if (wg < kNW) {
             const int eq = warp & 3;            // TMEM lane quarter
-            const int wtid = threadIdx.x - (kWarpA + 4 * wg) * 32;  // 0 .. 127
             const int col0 = wg * kCols;
             const uint32_t lane_base = static_cast<uint32_t>(eq * 32) << 16;
-            uint64_t* gbar = &group[wg];
-            uint32_t gphase = 0;
             int a_it = 0;
             bool ok = true;
             for (int it = 0; ok; ++it) {
@@ -554,12 +540,12 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
 #pragma unroll
                 for (int c = 0; c < kCols; ++c) m[c] = -nm[c];
                 if (!ok) break;
-                if (!item_sums(m, sm_, red_a[it & 1][wg], eq, lane, wtid, gbar, gphase,
-                               &pub_full[it & 1], &pub_empty[it & 1], (it >> 1) & 1,
-                               pub_s[it & 1] + col0, abort, lim)) {
-                    ok = false;
-                    break;
-                }
+                warp_sums(m, sm_, lane);
+                ok = __all_sync(0xffffffffu, mbar_wait(pub_empty, (it & 1) ^ 1, abort, lim));
+                if (!ok) break;
+                sums_s[eq * N + col0 + lane] = make_float2(m[0], sm_[0]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(pub_full);
             }
             if (!ok) {
                 *abort = 1;
@@ -605,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                     }
                 }
             }
-            if (!group_sync(&group[2], gphase, abort, lim) || *abort) {
+            if (!group_sync(group, gphase, abort, lim) || *abort) {
                 ok = false;
                 break;
             }
@@ -621,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                     (bits & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull)));
                 nlse_s[c] = real && v > 0.0 ? -(static_cast<float>(ex) + lg2_approx(f)) : -INFINITY;
             }
-            if (!group_sync(&group[2], gphase, abort, lim)) {
+            if (!group_sync(group, gphase, abort, lim)) {
                 ok = false;
                 break;
             }
@@ -660,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                 }
             }
             // every warp is done with nlse_s before the next item's lse overwrites it
-            if (!group_sync(&group[2], gphase, abort, lim)) {
+            if (!group_sync(group, gphase, abort, lim)) {
                 ok = false;
                 break;
             }
@@ -682,7 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
 template <int N, int W_PAD>
 cudaError_t launch_one(const LayersParams& p, int grid, cudaStream_t stream) {
     auto kern = score_layers_kernel<N, W_PAD>;
-    constexpr int smem = LayersSmem<N>::kDynamic;
+    constexpr int smem = LayersSmem<N>::kBytes;
     static bool configured = false;  // benign race: the attribute call is idempotent
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

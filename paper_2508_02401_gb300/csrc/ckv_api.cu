@@ -790,6 +790,7 @@ SelectLaunch select_launch(const Plan& pl, const ckv_batch* b, int T, int T_keep
     L.max_len = 0;
     for (int s = 0; s < b->num_seqs; ++s) {
         const int len = b->cu_seqlens_host[s + 1] - b->cu_seqlens_host[s];
+        if (len > kSelectOwnRows && L.n_long++ < kSelMaxLongSeqs) L.long_seq[L.n_long - 1] = s;
         L.min_len = std::min(L.min_len, len);
         L.max_len = std::max(L.max_len, len);
     }
@@ -1178,8 +1179,8 @@ ckv_status prepare_layers(const ckv_config* cfg, int32_t n_layers, const ckv_lay
     off = round_up(off + units * kMaxCols * sizeof(double), kWsAlign);
     lw->counters = off;  // and, after them, the kernel's item counter
     off = round_up(off + (units + 1) * sizeof(int), kWsAlign);
-    lw->next_unit = off;  // the selection kernel's work counter
-    off = round_up(off + sizeof(int), kWsAlign);
+    lw->next_unit = off;  // the selection kernel's work counters and flags
+    off = round_up(off + static_cast<size_t>(select_counters(b->num_seqs * pls[0].Hkv)) * sizeof(int), kWsAlign);
     lw->scores.assign(n_layers, 0);
     lw->keys.assign(n_layers, 0);
     for (int i = 0; i < n_layers; ++i) {

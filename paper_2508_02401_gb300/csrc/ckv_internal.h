@@ -117,6 +117,8 @@ struct LayersLaunch {
 cudaError_t launch_score_layers(const LayersLaunch& L, cudaStream_t stream);
 long long wait_limit_cycles();  // the current limit of a bounded wait, in SM clock cycles
 
+constexpr int kSelectOwnRows = 1024;  // the multi-layer selection: rows that a unit's CTA copies itself
+constexpr int kSelMaxLongSeqs = 64;
 struct SelectLaunch {
     const float* scores;        // [n_sel, T]
     float* pooled;              // [H_kv, T]
@@ -146,6 +148,10 @@ struct SelectLaunch {
     int64_t tok_stride, head_stride;
     void* k_out;
     void* v_out;
+    // The multi-layer selection: the sequences of more than kSelectOwnRows tokens (the first
+    // kSelMaxLongSeqs of them; n_long counts all)
+    int n_long;
+    int long_seq[kSelMaxLongSeqs];
     // The multi-layer selection: the scores viewed as 16-float lines (score_map_lines), with
     // 64 bytes of readable padding after the last row; nullptr: no such view.
     const CUtensorMap* score_map;
@@ -162,9 +168,10 @@ cudaError_t launch_pool(const SelectLaunch& L, cudaStream_t stream);
 cudaError_t launch_select(const SelectLaunch& L, cudaStream_t stream);
 // The selections of several layers (one SelectLaunch each, pooling from their scores) in one
 // launch per 32 layers: keys[i] is a [H_kv, select_key_stride(T, S)] scratch of 8-byte slots
-// of layer i (each sequence's segment 32-byte aligned), next_unit a work counter (cleared by the
-// call).
+// of layer i (each sequence's segment 32-byte aligned), next_unit select_counters(S * H_kv) ints of
+// work counters and flags (cleared by the call).
 int select_key_stride(int T, int S);
+int select_counters(int units_per_layer);
 cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, int n_layers,
                                  int* next_unit, int grid, cudaStream_t stream);
 

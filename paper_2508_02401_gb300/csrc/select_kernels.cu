@@ -148,6 +148,14 @@ struct SelectParams {
     int16_t group_first[kMaxQHeads + 1];
 };
 
+__device__ __forceinline__ void st_release(int* p, int v) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ int atomic_add_acq_rel(int* p, int v) {
     int old;
     asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
@@ -490,15 +498,16 @@ __device__ __noinline__ void copy_rows(const SelectParams& p, const UnitGeo& u, 
 }
 
 // Writes list[0..m) (sequence-local positions, in order) to the index rows at offset out_off
-// of the unit's kept tokens, and copies the K/V rows when asked, for KV heads [kv0, kv1) of
-// those the unit's selection serves: its own (per-KV-head scope) or all of them (per-layer
-// scope).
+// of the unit's kept tokens, and copies the K/V rows of the unit's first `own` kept tokens when
+// asked, for KV heads [kv0, kv1) of those the unit's selection serves: its own (per-KV-head scope)
+// or all of them (per-layer scope).
 __device__ __forceinline__ void emit_kept(const SelectParams& p, const UnitGeo& u, const int* list,
-                                          int m, int out_off, int kv0, int kv1) {
+                                          int m, int out_off, int kv0, int kv1, int own = INT_MAX) {
     for (int kv = kv0; kv < kv1; ++kv) {
         int32_t* out = p.idx + static_cast<size_t>(kv) * p.T_keep + u.keep_off + out_off;
         for (int e = threadIdx.x; e < m; e += blockDim.x) out[e] = list[e];
-        if (p.k) copy_rows(p, u, kv, list, m, u.keep_off + out_off);
+        const int rows = min(m, own - out_off);
+        if (p.k && rows > 0) copy_rows(p, u, kv, list, rows, u.keep_off + out_off);
     }
 }
 
@@ -1235,7 +1244,9 @@ __device__ __forceinline__ void pool_any_tma(const float* row, int d, int t, int
 //      among keys equal to the threshold is their rank by position, in shared memory when at
 //      most kLsTies were gathered, else by a scan of the list (which is in position order);
 //  (C) writes the kept candidates' positions in order (a block scan per kLsChunk of the list)
-//      with their K/V rows, and appends the window.
+//      with the K/V rows of the first `own`, and appends the window.
+// When no unit is left, the CTAs take the row copies that the units left, in jobs of kLsJob rows,
+// each once its unit has released its positions.
 // The same keys, ties and order as select_unit_kernel and the chunked kernels.
 constexpr int kLsThreads = 512;
 constexpr int kLsPer = 16;
@@ -1253,14 +1264,24 @@ constexpr int kLsAhead = 2;     // score-row chunks asked into L2 ahead of the o
 constexpr int kLsCand = 2048;   // keys sharing the k-th key's first digit gathered in shared memory
 constexpr int kLsTies = 256;    // keys equal to the k-th key ranked by position in shared memory
 constexpr int kSelMaxLayers = 32;
+// kSelectOwnRows kept rows of a unit are copied by the CTA that selects them; the rest are cut into jobs of kLsJob rows
+// that the CTAs take once no unit is left, so that a large budget's rows (3072 of them took one SM
+// 80 us) spread over the GPU.  Selection and copies, us a call, own rows 256 / 512 / 1024 / all:
+// 32 layers at L = 32768, budgets up to 3072: 144 / 139 / 133 / 159; 8 ragged layers with the lse
+// given, budgets up to 1536, whole calls: 288 / 283 / 290 / 295.
+constexpr int kLsJob = 256;
 
 struct SelectLayersParams {
     CUtensorMap score_map[kSelMaxLayers];  // each layer's scores as 16-float lines (map_mask)
     uint32_t map_mask;                     // bit i: score_map[i] is set
     SelectParams layer[kSelMaxLayers];
     uint2* cands[kSelMaxLayers];     // per layer [n_vec, key_stride]: (key, position) candidates
-    int* next_unit;                  // work counter, zero at launch
-    int n_layers, units_per_layer;   // units_per_layer = S * n_vec
+    int* next_unit;                  // work counters (units, then jobs), then a flag per unit; zero at launch
+    int n_layers, units_per_layer;   // units_per_layer = S * n_vec (S * H_kv with one selection per layer)
+    int own;                         // kept rows of a unit that its CTA copies itself
+    int job0[kSelMaxLayers + 1];     // first row-copy job of each layer
+    int unit_jobs[kSelMaxLayers];    // jobs of each unit of a long sequence
+    int long_seq[kSelMaxLongSeqs];   // the sequences of more than `own` tokens (where there are jobs)
     int key_stride;                  // select_key_stride(T, S)
 };
 
@@ -1289,8 +1310,14 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         if (seqlens_hash(p0.cu_seqlens, p0.S) != p0.cu_hash) record_error(p0.status, kDevBadSeqlens, 240);
     }
     const int n_units = P.n_layers * P.units_per_layer;
+    int* const unit_done = P.next_unit + 2;  // 1: the unit's positions are written, 2: it failed
+    int prev = -1, prev_state = 2;           // the last unit, if jobs wait for it
     for (;;) {
-        if (tid == 0) s_unit = atomicAdd(P.next_unit, 1);
+        if (tid == 0) {
+            // every thread's writes of the last unit precede the barrier that ended it
+            if (prev >= 0) st_release(unit_done + prev, prev_state);
+            s_unit = atomicAdd(P.next_unit, 1);
+        }
         fence_proxy_async_smem();  // this thread's writes to the stage before the unit's TMA loads
         __syncthreads();
         const int gu = s_unit;
@@ -1298,6 +1325,8 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         if (gu >= n_units) break;
         const int li = gu / P.units_per_layer, lu = gu % P.units_per_layer;
         const SelectParams& p = P.layer[li];
+        prev = P.unit_jobs[li] > 0 ? gu : -1;
+        prev_state = 2;
         // One selection per layer (n_vec = 1) is made by H_kv units, each writing the positions
         // and copying the rows of one KV head, so that the row copies spread over CTAs; every
         // copy of the selection is the same (the same inputs and steps).
@@ -1319,9 +1348,10 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
                     if (pooled) pooled[e0 + e] = 0.f;
                 }
                 __syncthreads();
-                emit_kept(p, u, list, m, e0, kv0, kv1);
+                emit_kept(p, u, list, m, e0, kv0, kv1, P.own);
                 __syncthreads();
             }
+            prev_state = 1;
             continue;
         }
         const int Pn = u.P, k = u.k;
@@ -1610,7 +1640,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
             int rk = block_excl_scan1<NT>(cnt, wsum[(b0 / kLsChunk) & 1], &tot);
             if (written + tot > k) break;  // checked below
             if (lcount + tot > kLsList) {  // block-uniform: write out the list first
-                emit_kept(p, u, list, lcount, lbase, kv0, kv1);
+                emit_kept(p, u, list, lcount, lbase, kv0, kv1, P.own);
                 lbase += lcount;
                 lcount = 0;
                 __syncthreads();
@@ -1633,15 +1663,53 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         }
         if (lcount + p.w > kLsList) {
             __syncthreads();
-            emit_kept(p, u, list, lcount, lbase, kv0, kv1);
+            emit_kept(p, u, list, lcount, lbase, kv0, kv1, P.own);
             lbase += lcount;
             lcount = 0;
             __syncthreads();
         }
         for (int i = tid; i < p.w; i += NT) list[lcount + i] = Pn + i;
         __syncthreads();
-        emit_kept(p, u, list, lcount + p.w, lbase, kv0, kv1);
+        emit_kept(p, u, list, lcount + p.w, lbase, kv0, kv1, P.own);
         __syncthreads();
+        prev_state = 1;
+    }
+    // Row copies that the units left: every unit has been taken by a CTA that runs and waits for no
+    // other, so the waits below end.
+    const int n_jobs = P.job0[P.n_layers];
+    int* const list = reinterpret_cast<int*>(st);
+    for (;;) {
+        if (tid == 0) s_unit = atomicAdd(P.next_unit + 1, 1);
+        __syncthreads();
+        const int job = s_unit;
+        __syncthreads();
+        if (job >= n_jobs) break;
+        int li = 0;
+        while (P.job0[li + 1] <= job) ++li;
+        const SelectParams& p = P.layer[li];
+        const int q = (job - P.job0[li]) / P.unit_jobs[li];  // (long sequence, KV head)
+        const int row0 = P.own + (job - P.job0[li]) % P.unit_jobs[li] * kLsJob;
+        const int kv = q % p.Hkv, lu = P.long_seq[q / p.Hkv] * p.Hkv + kv;
+        UnitGeo u;
+        if (!unit_geo(p, p.n_vec == 1 ? lu / p.Hkv : lu, u)) continue;
+        const int m = min(kLsJob, u.n_keep - row0);
+        if (m <= 0) continue;
+        if (tid == 0) {
+            const int* flag = unit_done + li * P.units_per_layer + lu;
+            const long long t0 = clock64();
+            int f;
+            while ((f = ld_acquire_gpu(flag)) == 0 && clock64() - t0 <= kWaitTimeoutCycles) __nanosleep(64);
+            if (f == 0) record_error(p.status, kDevTimeout, 251);
+            s_cnt = f;
+        }
+        __syncthreads();
+        if (s_cnt == 1) {
+            const int32_t* src = p.idx + static_cast<size_t>(kv) * p.T_keep + u.keep_off + row0;
+            for (int e = tid; e < m; e += NT) list[e] = min(max(__ldcg(src + e), 0), u.L - 1);
+        }
+        __syncthreads();
+        if (s_cnt == 1) copy_rows(p, u, kv, list, m, u.keep_off + row0);
+        __syncthreads();  // the list and s_cnt are read
     }
 }
 
@@ -1777,6 +1845,8 @@ cudaError_t launch_gather(const GatherLaunch& L, cudaStream_t stream) {
 // 8-byte (key, position) slots per layer.  One launch per
 // kSelMaxLayers layers; `next_unit` (kSelMaxLayers-aligned count of ints) is the work counter
 // of each launch and is cleared first.
+int select_counters(int units_per_layer) { return 2 + kSelMaxLayers * units_per_layer; }
+
 int select_key_stride(int T, int S) { return (T + 4 * S + 3) & ~3; }
 
 cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, int n_layers,
@@ -1841,7 +1911,29 @@ cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, 
         P.next_unit = next_unit;
         const int units = nl * P.units_per_layer;
         if (units == 0) continue;
-        cudaError_t e = cudaMemsetAsync(next_unit, 0, sizeof(int), stream);
+        // Row-copy jobs, unless so many sequences are long that the units themselves spread the rows.
+        const int n_long = Ls[l0].n_long;
+        long long jobs = 0;
+        P.own = INT_MAX;
+        if (n_long > 0 && n_long <= kSelMaxLongSeqs) {
+            for (int i = 0; i < n_long; ++i) P.long_seq[i] = Ls[l0].long_seq[i];
+            for (int i = 0; i < nl; ++i) {
+                const SelectLaunch& L = Ls[order[i]];
+                const int rows = L.k ? std::min(L.budget, L.max_len) : 0;
+                P.unit_jobs[i] = rows > kSelectOwnRows ? (rows - kSelectOwnRows + kLsJob - 1) / kLsJob : 0;
+                jobs += static_cast<long long>(P.unit_jobs[i]) * n_long * L.Hkv;
+                if (jobs > (1 << 30)) break;
+                P.job0[i + 1] = static_cast<int>(jobs);
+            }
+        }
+        if (jobs > 0 && jobs <= (1 << 30)) {
+            P.own = kSelectOwnRows;
+        } else {
+            memset(P.unit_jobs, 0, sizeof P.unit_jobs);
+            memset(P.job0, 0, sizeof P.job0);
+        }
+        const int counters = P.own == INT_MAX ? 2 : select_counters(P.units_per_layer);
+        cudaError_t e = cudaMemsetAsync(next_unit, 0, static_cast<size_t>(counters) * sizeof(int), stream);
         if (e != cudaSuccess) return e;
         NvtxRange range("select_layers_kernel");
         select_layers_kernel<<<std::min(grid, units), kLsThreads, kLsSmem, stream>>>(P);

@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
 // position base-4 on, so element e of the row sits at position base-4-d+e, d = the offset of
 // position base-4 in its line.  The TMA writes each 64-byte line with the 64-byte swizzle: the
 // 16-byte chunk bits 4-5 of a byte offset XOR its bits 7-8 (rows 1024-byte aligned).  For the
-// pooling's reads of 16 elements per thread that places the 16-byte reads of every
+// pooling's reads of 8 (or 16) elements per thread that places the 16-byte reads of every
 // quarter-warp in distinct bank groups.
 constexpr int kLsTmaBoxes = 3;
 constexpr int kLsTmaRow = kLsTmaBoxes * kScoreMapBoxLines * 16;   // floats per stage row
@@ -1143,19 +1143,19 @@ __device__ __forceinline__ int stage_offset(size_t T, int t0, int r, int base) {
     return f >= 0 ? static_cast<int>(f & 15) : static_cast<int>(f + 16);
 }
 
-// Pools the PER = 16 outputs of thread t (positions base+16t .. base+16t+15) from one stage
-// row: its 24 elements d+16t .. d+16t+23 (positions base-4+16t ..), d = 4a + SHIFT, in six
-// 16-byte reads from element 4a+16t on (seven when SHIFT > 0), those outside [0, P) taken as
-// zero; output i covers elements 16t+i+4-HALF .. 16t+i+4+HALF.  The same arithmetic, in the
+// Pools the PER outputs of thread t (positions base+PER t ..) from one stage row: its PER + 8
+// elements from d + PER t on (positions base-4+PER t ..), d = 4a + SHIFT, in 16-byte reads from
+// element 4a + PER t on (one more when SHIFT > 0), those outside [0, P) taken as zero; output i
+// covers elements PER t+i+4-HALF .. PER t+i+4+HALF.  The same arithmetic, in the
 // same order, as pool_window.
 template <int HALF, int SHIFT, int PER>
 __device__ __forceinline__ void pool_window_tma(const float* row, int d, int t, int nvalid, bool is_max,
                                                 float kf, int pos0, int P, float (&acc)[PER]) {
-    static_assert(PER == 16 && HALF >= 0 && HALF <= 4 && SHIFT >= 0 && SHIFT < 4, "window");
-    constexpr int kReads = SHIFT > 0 ? 7 : 6;
+    static_assert(PER % 8 == 0 && HALF >= 0 && HALF <= 4 && SHIFT >= 0 && SHIFT < 4, "window");
+    constexpr int kElems = PER + 8, kReads = kElems / 4 + (SHIFT > 0 ? 1 : 0);
     float r[4 * kReads];
     const char* rb = reinterpret_cast<const char*>(row);
-    const int e0 = (d & ~3) + 16 * t;
+    const int e0 = (d & ~3) + PER * t;
 #pragma unroll
     for (int q = 0; q < kReads; ++q) {
         const float4 x = *reinterpret_cast<const float4*>(rb + sw64(4 * (e0 + 4 * q)));
@@ -1164,21 +1164,21 @@ __device__ __forceinline__ void pool_window_tma(const float* row, int d, int t, 
         r[4 * q + 2] = x.z;
         r[4 * q + 3] = x.w;
     }
-    float w[24];
+    float w[kElems];
 #pragma unroll
-    for (int j = 0; j < 24; ++j) w[j] = r[SHIFT + j];
-    const int p0 = pos0 + 16 * t;  // position of w[0]
-    if (p0 < 0 || p0 + 24 > P) {
+    for (int j = 0; j < kElems; ++j) w[j] = r[SHIFT + j];
+    const int p0 = pos0 + PER * t;  // position of w[0]
+    if (p0 < 0 || p0 + kElems > P) {
 #pragma unroll
-        for (int j = 0; j < 24; ++j)
+        for (int j = 0; j < kElems; ++j)
             if (p0 + j < 0 || p0 + j >= P) w[j] = 0.f;
     }
     if (is_max) {
         // maxima of three neighbours, shared by the windows that contain them (a maximum is
         // exact in any order)
-        float m3[22];
+        float m3[kElems - 2];
 #pragma unroll
-        for (int j = 0; j < 22; ++j) m3[j] = fmax3(w[j], w[j + 1], w[j + 2]);
+        for (int j = 0; j < kElems - 2; ++j) m3[j] = fmax3(w[j], w[j + 1], w[j + 2]);
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             if (i < nvalid) {
@@ -1248,8 +1248,11 @@ __device__ __forceinline__ void pool_any_tma(const float* row, int d, int t, int
 // When no unit is left, the CTAs take the row copies that the units left, in jobs of kLsJob rows,
 // each once its unit has released its positions.
 // The same keys, ties and order as select_unit_kernel and the chunked kernels.
-constexpr int kLsThreads = 512;
-constexpr int kLsPer = 16;
+// 32 warps of 8 positions a thread: the phases wait on barriers and shared-memory round trips, which
+// the extra warps fill (16 warps of 16 positions: 588 -> 572 us a call of 32 layers at L = 32768,
+// 473 -> 456 with the lse given, 1963 -> 1951 at L = 131072).
+constexpr int kLsThreads = 1024;
+constexpr int kLsPer = 8;
 constexpr int kLsChunk = kLsThreads * kLsPer;                    // 8192 positions
 constexpr int kLsStageFloats = kLsChunk + 2 * kMaxHalo;
 constexpr int kLsStageLoads = (kLsStageFloats + kLsThreads - 1) / kLsThreads;
@@ -1268,8 +1271,8 @@ constexpr int kSelMaxLayers = 32;
 // that the CTAs take once no unit is left, so that a large budget's rows (3072 of them took one SM
 // 80 us) spread over the GPU.  Selection and copies, us a call, own rows 256 / 512 / 1024 / all:
 // 32 layers at L = 32768, budgets up to 3072: 144 / 139 / 133 / 159; 8 ragged layers with the lse
-// given, budgets up to 1536, whole calls: 288 / 283 / 290 / 295.
-constexpr int kLsJob = 256;
+// given, budgets up to 1536, whole calls: 288 / 283 / 290 / 295 (with 512 threads and jobs of 256 rows).
+constexpr int kLsJob = 512;
 
 struct SelectLayersParams {
     CUtensorMap score_map[kSelMaxLayers];  // each layer's scores as 16-float lines (map_mask)
@@ -1368,7 +1371,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         // chunk's rows are copied in while this chunk is pooled (two buffers of nr rows).
         const int half = p.pool_kernel >> 1;
         const int r0 = p.group_first[u.g], nr = p.group_first[u.g + 1] - r0;
-        // TMA staging when the pooling window fits a thread's 24 staged elements and the unit's
+        // TMA staging when the pooling window fits a thread's PER + 8 staged elements and the unit's
         // rows fit the stage, in two buffers (the next chunk loaded while this one is pooled)
         // or else one; otherwise 4-byte copies in the padded layout
         const bool tma = ((P.map_mask >> li) & 1u) && p.from_scores && p.head_order == 0 && half <= 4 &&
@@ -1485,10 +1488,12 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
                 for (int i = 0; i < PER; ++i) cnt += (i < nvalid && (key[i] >> kHistShift) >= lo) ? 1 : 0;
                 int tot;
                 int off = n_cand + block_excl_scan1<NT>(cnt, wsum[c & 1], &tot);
+                if (cnt > 0) {
 #pragma unroll
-                for (int i = 0; i < PER; ++i)
-                    if (i < nvalid && (key[i] >> kHistShift) >= lo)
-                        cands[off++] = make_uint2(key[i], static_cast<uint32_t>(base + jb + i));
+                    for (int i = 0; i < PER; ++i)
+                        if (i < nvalid && (key[i] >> kHistShift) >= lo)
+                            cands[off++] = make_uint2(key[i], static_cast<uint32_t>(base + jb + i));
+                }
                 n_cand += tot;
             }
             if (piped) __syncthreads();  // every thread is done with this chunk's buffer
@@ -1613,7 +1618,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
             int cnt = 0, pos[PER];
 #pragma unroll
             for (int q = 0; q < PER / 2; ++q) {
-                // 16-byte loads: the list is 32-byte aligned, b0 + jb a multiple of 16
+                // 16-byte loads: the list is 32-byte aligned, b0 + jb a multiple of PER
                 uint4 x2 = make_uint4(0u, 0u, 0u, 0u);
                 if (2 * q < nvalid) {
                     if (2 * q + 1 < nvalid) {

@@ -112,7 +112,6 @@ constexpr int kUnitThreads = 1024;           // select_unit_kernel
 constexpr int kUnitPer = 16;
 constexpr int kUnitLen = kUnitThreads * kUnitPer;
 constexpr int kUnitStage = kUnitLen + 2 * kMaxHalo;
-constexpr int kUnitStageLoads = (kUnitStage + kUnitThreads - 1) / kUnitThreads;
 constexpr int kUnitCandMax = 1024;            // first-digit ties ranked pairwise up to this many
 static_assert(kWarpSpan % 32 == 0 && (1 << kChunkShift) == kChunk, "chunk shape");
 
@@ -512,13 +511,18 @@ __device__ __forceinline__ void emit_kept(const SelectParams& p, const UnitGeo& 
 }
 
 // ------------------------------------------------------------------ units of up to kUnitLen
+// PER positions per thread: the smallest of 2, 4, 8 and 16 that covers the batch's longest such unit,
+// so that every warp has a share of the pooling, the counts and the scans (with 16 throughout, a unit
+// of 2048 tokens left 28 of 32 warps idle).
+template <int PER>
 __global__ void __launch_bounds__(kUnitThreads, 1) select_unit_kernel(const __grid_constant__ SelectParams p) {
     extern __shared__ __align__(16) float ust[];  // pooling stage, then the kept list
     __shared__ int hist[kHistBins];
     __shared__ int scratch[33];
     __shared__ int s_digit, s_above, s_cut, s_cnt;
     __shared__ uint32_t s_thr;
-    constexpr int NT = kUnitThreads, PER = kUnitPer;
+    constexpr int NT = kUnitThreads;
+    constexpr int kLoads = (NT * PER + 2 * kMaxHalo + NT - 1) / NT;
     // A selection that serves several KV heads (per-layer scope) is made by one block per KV
     // head, each gathering its own head's rows: the selection is recomputed (from L2-resident
     // scores) rather than one block copying every head's rows alone.
@@ -528,7 +532,7 @@ __global__ void __launch_bounds__(kUnitThreads, 1) select_unit_kernel(const __gr
         record_error(p.status, kDevBadSeqlens, 230);
     UnitGeo u;
     if (!unit_geo(p, unit, u)) return;
-    if (u.L > kUnitLen) return;  // a long unit: the chunked kernels take it
+    if (u.L > NT * PER) return;  // a long unit: the chunked kernels take it
     const int kv = u.g * per + sub;  // the KV head whose rows this block writes
     if (u.g == 0 && sub == 0 && tid == 0) {
         p.cu_keep[u.s + 1] = u.keep_off + u.n_keep;
@@ -551,7 +555,7 @@ __global__ void __launch_bounds__(kUnitThreads, 1) select_unit_kernel(const __gr
         for (int j = P + tid; j < u.L; j += NT) pooled[j] = 0.f;
     const int jb = tid * PER, nvalid = P - jb;
     float acc[PER];
-    pooled_values<NT, PER, kUnitStageLoads, stage_words(kUnitStage)>(p, u, ust, 0, P, acc);
+    pooled_values<NT, PER, kLoads, stage_words(kUnitStage)>(p, u, ust, 0, P, acc);
     if (zeros)
 #pragma unroll
         for (int i = 0; i < PER; ++i)
@@ -1790,8 +1794,9 @@ cudaError_t launch_select(const SelectLaunch& L, cudaStream_t stream) {
     if (!configured) {
         e = cudaFuncSetAttribute(compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCompactSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(select_unit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUnitSmem);
-        if (e != cudaSuccess) return e;
+        for (auto kern : {select_unit_kernel<2>, select_unit_kernel<4>, select_unit_kernel<8>, select_unit_kernel<16>})
+            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kUnitSmem)) != cudaSuccess)
+                return e;
         configured = true;
     }
     if (sel_smem > sel_smem_set) {
@@ -1802,7 +1807,11 @@ cudaError_t launch_select(const SelectLaunch& L, cudaStream_t stream) {
     }
     if (L.min_len <= kUnitLen) {
         NvtxRange range("select_unit_kernel");
-        select_unit_kernel<<<units * (L.Hkv / L.n_vec), kUnitThreads, kUnitSmem, stream>>>(p);
+        auto kern = L.max_len <= 2 * kUnitThreads   ? select_unit_kernel<2>
+                    : L.max_len <= 4 * kUnitThreads ? select_unit_kernel<4>
+                    : L.max_len <= 8 * kUnitThreads ? select_unit_kernel<8>
+                                                    : select_unit_kernel<16>;
+        kern<<<units * (L.Hkv / L.n_vec), kUnitThreads, kUnitSmem, stream>>>(p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (L.max_len > kUnitLen) {

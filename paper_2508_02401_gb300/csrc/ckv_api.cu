@@ -286,7 +286,9 @@ ckv_status plan_score_stream(const Plan& pl, const ckv_batch* b, int skip_le, in
     struct RawUnit {
         int seq, start, len, batch, tiles;
     };
-    std::vector<RawUnit> raw;
+    // (kept between calls of a thread: a call allocates only where it plans more than any before)
+    static thread_local std::vector<RawUnit> raw;
+    raw.clear();
     int64_t total = 0;
     for (int s = 0; s < b->num_seqs; ++s) {
         const int t0 = b->cu_seqlens_host[s];
@@ -311,39 +313,47 @@ ckv_status plan_score_stream(const Plan& pl, const ckv_batch* b, int skip_le, in
         int raw;         // index into raw
         ScoreItem item;  // unit filled in per slice
     };
-    std::vector<std::vector<Run>> runs(grid);
+    // the runs of CTA c are runs[first[c]] .. runs[first[c + 1] - 1]
+    static thread_local std::vector<Run> runs;
+    static thread_local std::vector<int> first;
+    runs.clear();
+    first.assign(1, 0);
     int cta = 0;
     int64_t filled = 0;
     for (int ui = 0; ui < static_cast<int>(raw.size()); ++ui) {
         for (int t = 0; t < raw[ui].tiles;) {
             const int take = static_cast<int>(std::min<int64_t>(raw[ui].tiles - t, per - filled));
-            runs[cta].push_back({ui, ScoreItem{0, static_cast<uint16_t>(take), static_cast<uint32_t>(t)}});
+            runs.push_back({ui, ScoreItem{0, static_cast<uint16_t>(take), static_cast<uint32_t>(t)}});
             t += take;
             filled += take;
             if (filled == per && cta + 1 < grid) {
                 ++cta;
                 filled = 0;
+                first.push_back(static_cast<int>(runs.size()));
             }
         }
     }
-    size_t rounds = 0;
-    for (const auto& r : runs) rounds = std::max(rounds, r.size());
+    first.resize(grid + 1, static_cast<int>(runs.size()));
+    int rounds = 0;
+    for (int c = 0; c < grid; ++c) rounds = std::max(rounds, first[c + 1] - first[c]);
+    auto has = [&](int c, int r) { return r < first[c + 1] - first[c]; };
     L.grid = grid;
     const int max_rounds = std::max(1, max_items_per_launch / grid);
-    std::vector<int> local(raw.size(), -1);
-    size_t r = 0;
+    static thread_local std::vector<int> local, used;
+    local.assign(raw.size(), -1);
+    int r = 0;
     while (r < rounds) {
         ScoreSlice sl{static_cast<int>(L.items.size()), 0, static_cast<int>(L.units.size()), 0};
-        std::vector<int> used;
+        used.clear();
         while (r < rounds && sl.n_rounds < max_rounds) {
             int fresh = 0;
             for (int c = 0; c < grid; ++c)
-                if (r < runs[c].size() && local[runs[c][r].raw] < 0) ++fresh;  // an upper bound
+                if (has(c, r) && local[runs[first[c] + r].raw] < 0) ++fresh;  // an upper bound
             if (sl.n_rounds > 0 && sl.n_units + fresh > kMaxScoreUnits) break;
             for (int c = 0; c < grid; ++c) {
                 ScoreItem it{0, 0, 0};
-                if (r < runs[c].size()) {
-                    const int ui = runs[c][r].raw;
+                if (has(c, r)) {
+                    const int ui = runs[first[c] + r].raw;
                     if (local[ui] < 0) {
                         if (sl.n_units >= kMaxScoreUnits)
                             return fail(CKV_ERR_UNSUPPORTED, "too many scoring units in a round");
@@ -358,7 +368,7 @@ ckv_status plan_score_stream(const Plan& pl, const ckv_batch* b, int skip_le, in
                         su.nitems = 0;
                         L.units.push_back(su);
                     }
-                    it = runs[c][r].item;
+                    it = runs[first[c] + r].item;
                     it.unit = static_cast<uint16_t>(local[ui]);
                 }
                 L.items.push_back(it);

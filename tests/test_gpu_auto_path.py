@@ -1,0 +1,50 @@
+"""The automatic choice of the one-layer scoring kernel at N = 64: small calls take the TMEM-resident
+kernel, larger ones the two-pass kernel.  Around the limits of the rule (key tiles and units per CTA),
+with both layouts of K, the scores agree with the two-pass kernel's and the layer with the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import ckv_synth as cs
+import oracle
+import paper_2508_02401_gb300 as ckv
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+# 8 groups: 608 tiles of 152 CTAs is 76 per unit (9728 tokens); 76 units is 9 sequences
+CASES = [((130,), 2), ((2048,), 2), ((9728,), 2), ((9729,), 2), ((700,) * 9, 2), ((500,) * 10, 2),
+         ((4000, 33, 1, 3000), 2), ((1500,), 4)]
+
+
+@pytest.mark.parametrize("interleaved", [False, True])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_small_calls_agree_with_the_two_pass_kernel(case, interleaved):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    ckv.load()
+    oracle.build()
+    lens, heads = CASES[case]
+    wl = cs.Workload(name="auto", num_layers=1, num_q_heads=32, num_kv_heads=8, seqlens=lens, window=32,
+                     heads_per_group=heads, budget_mean=100, budget_uniform=True, outlier_channels=8, seed=91)
+    li = wl.layer(0)
+    if not interleaved:
+        gu.check_layer(wl, 0, li, gu.run_gpu(wl, 0, li), gu.run_oracle(wl, 0, li))
+    batch = ckv.Batch(wl.cu_seqlens())
+    q, k = gu.to_dev(li.q_win), gu.to_dev(li.k)
+    strides = {}
+    if interleaved:
+        k = torch.stack([k, torch.zeros_like(k)], dim=1).contiguous()[:, 0]
+        strides = dict(tok_stride=2 * 8 * 128, head_stride=128)
+    got = []
+    for path in (ckv.SCORE_AUTO, ckv.SCORE_RELOAD):
+        cfg = ckv.Config.from_workload(wl, score_path=path)
+        _, n_sel = ckv.ckv_keep_lengths(cfg, 0, batch)
+        sc = gu.Guarded((n_sel, batch.total_tokens), torch.float32, float("nan"))
+        ws = ckv.new_workspace(cfg, 0, batch)
+        ckv.ckv_score_window(cfg, 0, batch, q, k, sc.view, ws, **strides)
+        assert ckv.ckv_read_device_status(ws) == (0, 0)
+        sc.check()
+        got.append(sc.view.cpu().numpy().astype(np.float64))
+    # each side is within 1e-3 of the oracle (fp32 logits of up to about 40 in base-2 units: 2e-5)
+    gu.assert_close_rows(got[0], got[1], rtol=1e-4)

@@ -513,7 +513,8 @@ __device__ __forceinline__ void emit_kept(const SelectParams& p, const UnitGeo& 
 // ------------------------------------------------------------------ units of up to kUnitLen
 // PER positions per thread: the smallest of 2, 4, 8 and 16 that covers the batch's longest such unit,
 // so that every warp has a share of the pooling, the counts and the scans (with 16 throughout, a unit
-// of 2048 tokens left 28 of 32 warps idle).
+// of 2048 tokens left 28 of 32 warps idle).  GPU time of a call: one layer of 2048 tokens 28.7 ->
+// 23.5 us, of 8191 tokens with the lse given 26.7 -> 22.6; above 8192 tokens it is 16 as before.
 template <int PER>
 __global__ void __launch_bounds__(kUnitThreads, 1) select_unit_kernel(const __grid_constant__ SelectParams p) {
     extern __shared__ __align__(16) float ust[];  // pooling stage, then the kept list
@@ -1284,7 +1285,8 @@ struct SelectLayersParams {
     SelectParams layer[kSelMaxLayers];
     uint2* cands[kSelMaxLayers];     // per layer [n_vec, key_stride]: (key, position) candidates
     int* next_unit;                  // work counters (units, then jobs), then a flag per unit; zero at launch
-    int n_layers, units_per_layer;   // units_per_layer = S * n_vec (S * H_kv with one selection per layer)
+    int n_layers, units_per_layer;   // units_per_layer = S * n_vec (S * copies with one selection per layer)
+    int copies, heads;               // one selection per layer: units that make it, KV heads each serves
     int own;                         // kept rows of a unit that its CTA copies itself
     int job0[kSelMaxLayers + 1];     // first row-copy job of each layer
     int unit_jobs[kSelMaxLayers];    // jobs of each unit of a long sequence
@@ -1334,13 +1336,13 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         const SelectParams& p = P.layer[li];
         prev = P.unit_jobs[li] > 0 ? gu : -1;
         prev_state = 2;
-        // One selection per layer (n_vec = 1) is made by H_kv units, each writing the positions
-        // and copying the rows of one KV head, so that the row copies spread over CTAs; every
+        // One selection per layer (n_vec = 1) is made by `copies` units, each writing the positions
+        // and copying the rows of `heads` KV heads, so that the row copies spread over CTAs; every
         // copy of the selection is the same (the same inputs and steps).
-        const int copies = p.n_vec == 1 ? p.Hkv : 1, cu = lu % copies, unit = lu / copies;
+        const int copies = P.copies, cu = lu % copies, unit = lu / copies;
         UnitGeo u;
         if (!unit_geo(p, unit, u)) continue;
-        const int kv0 = p.n_vec == p.Hkv ? u.g : cu, kv1 = kv0 + 1;
+        const int kv0 = p.n_vec == p.Hkv ? u.g : cu * P.heads, kv1 = min(kv0 + P.heads, p.Hkv);
         if (u.g == 0 && cu == 0 && tid == 0) {
             p.cu_keep[u.s + 1] = u.keep_off + u.n_keep;
             if (u.s == 0) p.cu_keep[0] = 0;
@@ -1698,9 +1700,10 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
         const SelectParams& p = P.layer[li];
         const int q = (job - P.job0[li]) / P.unit_jobs[li];  // (long sequence, KV head)
         const int row0 = P.own + (job - P.job0[li]) % P.unit_jobs[li] * kLsJob;
-        const int kv = q % p.Hkv, lu = P.long_seq[q / p.Hkv] * p.Hkv + kv;
+        const int kv = q % p.Hkv, seq = P.long_seq[q / p.Hkv];
+        const int lu = p.n_vec == p.Hkv ? seq * p.Hkv + kv : seq * P.copies + kv / P.heads;
         UnitGeo u;
-        if (!unit_geo(p, p.n_vec == 1 ? lu / p.Hkv : lu, u)) continue;
+        if (!unit_geo(p, p.n_vec == p.Hkv ? lu : seq, u)) continue;
         const int m = min(kLsJob, u.n_keep - row0);
         if (m <= 0) continue;
         if (tid == 0) {
@@ -1863,6 +1866,47 @@ int select_counters(int units_per_layer) { return 2 + kSelMaxLayers * units_per_
 
 int select_key_stride(int T, int S) { return (T + 4 * S + 3) & ~3; }
 
+// KV heads that a unit serves with one selection per layer.  More of them repeat the selection less
+// often but copy more rows each, so it is the number whose units, dealt to the grid in order (the
+// largest budgets first), take least time: at least their sum over the grid, the first unit, and for
+// every full round j + 1 units of the size of the one that begins round j + 1.  A unit takes 16 us and
+// per 8192 positions 2 us and half of one a score row, and 17 ns a row copied (fitted to the figures
+// below).  GPU time of a call at 1 / 2 / 4 / 8 heads (8 KV heads, four score rows), us, the one taken first:
+//   32 layers of one prompt of 8192, budget 256:       2: 130    136 /  -  / 152 / 200
+//   24 layers of it:                                   1: 117     -  / 121 / 148 / 200
+//   8 layers of it:                                    1:  66     -  /  74 /  89 / 119
+//   32 layers of four prompts of 8192:                 4: 304    394 / 337 /  -  / 332
+//   32 layers of eight prompts of 2048:                8: 267    461 / 350 / 298 /  -
+//   32 layers of one prompt of 32768, budget 1024:     2: 343    351 /  -  / 392 / 502
+//   8 layers of one prompt of 131072, budget 1024:     1: 441     -  / 465 / 516 / 617
+int heads_per_unit(const SelectLaunch* Ls, const int* order, int nl, int grid) {
+    const int Hkv = Ls[order[0]].Hkv, S = Ls[order[0]].S;
+    if (S <= 0) return 1;
+    const int len = Ls[order[0]].T / S;
+    const float chunks = static_cast<float>((len + kLsChunk - 1) / kLsChunk);
+    int best = 1;
+    float best_us = 0.f;
+    for (int h = 1; h < 2 * Hkv; h *= 2) {
+        const long long per = static_cast<long long>(S) * ((Hkv + h - 1) / h);  // units of a layer
+        float t[kSelMaxLayers], us = 0.f;
+        for (int i = 0; i < nl; ++i) {
+            const SelectLaunch& L = Ls[order[i]];
+            const int rows = L.k ? std::min(std::min(L.budget, len), kSelectOwnRows) : 0;
+            t[i] = 16.f + chunks * (2.f + 0.5f * static_cast<float>(L.group_first[1])) +
+                   0.017f * static_cast<float>(std::min(h, Hkv)) * static_cast<float>(rows);
+            us += t[i] * static_cast<float>(per) / static_cast<float>(grid);
+        }
+        us = std::max(us, t[0]);
+        for (long long j = 1; j <= 64 && j * grid < per * nl; ++j)  // (past 64 rounds the sum decides)
+            us = std::max(us, static_cast<float>(j + 1) * t[j * grid / per]);
+        if (h == 1 || us < best_us) {
+            best_us = us;
+            best = std::min(h, Hkv);
+        }
+    }
+    return best;
+}
+
 cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, int n_layers,
                                  int* next_unit, int grid, cudaStream_t stream) {
     static SelectLayersParams P;  // ~25 KB; calls are serialised by `mu`
@@ -1920,7 +1964,12 @@ cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, 
             }
         }
         P.n_layers = nl;
-        P.units_per_layer = Ls[l0].S * Ls[l0].n_vec * (Ls[l0].n_vec == 1 ? Ls[l0].Hkv : 1);
+        P.copies = P.heads = 1;
+        if (Ls[l0].n_vec == 1) {
+            P.heads = heads_per_unit(Ls, order, nl, grid);
+            P.copies = (Ls[l0].Hkv + P.heads - 1) / P.heads;
+        }
+        P.units_per_layer = Ls[l0].S * Ls[l0].n_vec * P.copies;
         P.key_stride = select_key_stride(Ls[l0].T, Ls[l0].S);
         P.next_unit = next_unit;
         const int units = nl * P.units_per_layer;

@@ -1,4 +1,4 @@
-// Pieces shared by the two window-scoring kernels (score_kernel.cu, score_resident.cu): the
+// Pieces shared by the two window-scoring kernels (score_layers.cu, score_resident.cu): the
 // launch parameters, the warp roles' common constants and the epilogue arithmetic.
 #pragma once
 

@@ -1,5 +1,5 @@
 // Window-attention scoring with the logits resident in tensor memory (arxiv 2508.02401,
-// Sec. 3.3 with the attention of Eq. 2): the same scores as score_kernel.cu,
+// Sec. 3.3 with the attention of Eq. 2): the same scores as score_layers.cu,
 //
 //   a_h[j] = sum_{r < w, j <= P+r} exp(s_{h,r,j} - lse_{h,r}),   s_{h,r,j} = scale * q_{h,r}.k_j,
 //
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_resident_kernel(const __gri
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
-    // Registers as in score_kernel.cu: launched at 128 per thread; the control warpgroup gives
+    // Registers as in score_layers.cu: launched at 128 per thread; the control warpgroup gives
     // up to 56, the pass-1 warpgroups take 160, pass 2 keeps 128.
     const int R = p.n_rounds;
     const int G = gridDim.x;

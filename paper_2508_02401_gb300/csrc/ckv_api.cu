@@ -558,19 +558,66 @@ struct LayerJob {
     int64_t lse_stride = 0;
 };
 
-// The items of one launch of the two-pass kernel: unit (lb, s), of tiles[s] key tiles, is
-// split into m = ceil(tiles / c) items of balanced length, unit after unit (head batch major);
-// `units` ends with an entry holding the total.  c is kItemTiles, or more where a unit would
-// otherwise have more items than the launch has CTAs (the kernel's progress argument needs at
-// most G).  Items are long enough that their fixed costs (taking the item, loading its query
-// rows, publishing its sums, computing the unit's lse) are paid rarely, and short enough that
-// the faster SMs take more of the work and that the tiles pass 2 re-reads stay in L2.
+// Key tiles per item of a launch over n_lb head batches of sequences of tiles[s] key tiles.  At least
+// ceil(max_tiles / G), so that a unit has at most G items (the kernel's progress argument).
+//
+// A launch of many rounds of items: long enough that an item's fixed costs (taking it, loading its
+// query rows, publishing its sums, the unit's lse) are paid rarely, and short enough that the faster
+// SMs take more of the work and that the tiles pass 2 re-reads stay in L2.  Scoring, us a call, at 11 /
+// 12 / 13 / 14 / 16 tiles: 32 layers of 131072 tokens 1851 / 1878 / 1905 / 1814 / -; 16 of 65536
+// 447 / 428 / 434 / 445 / -; 32 of 32768 435 / 427 / 429 / 436 / 495; 28 ragged 830 / 828 / 837 / 841 / -;
+// 32 of 16384 230 / 228 / 228 / 227 / -; 32 of 8192 - / 130 / 130 / 129 / 143.
+//
+// A launch of few rounds lasts its rounds times the longest item (a tile takes about 0.9 us from its
+// load to its score, the two passes hardly overlap), a fixed cost a round of about two tiles, and a
+// tail of about a quarter of an item; the length that makes this least is taken, so that the items
+// fill whole rounds.  14 tiles -> this rule, us a call: one layer of 8192 / 16384 / 32768 / 65536 tokens
+// 26.7 -> 18.6 / 26.7 -> 20.8 / 28.6 (14 tiles) / 49.7 -> 47.1; of 8192 tokens 2 layers 28.9 -> 24.6,
+// 4 layers 37.1 -> 30.8, 8 layers 52.7 -> 49.0; with the lse given 43.0 -> 41.2, -, 62.7 -> 59.8 (with
+// the selection).  More units than CTAs, or more than six rounds, even out by themselves.
 constexpr int kItemTiles = 14;
+constexpr int kMidItemTiles = 12;                      // where the longest sequence has
+constexpr int kMidFrom = 160, kMidTo = 512;            // this many tiles
+constexpr int kFewRounds = 6, kMaxItemTiles = 16;
+int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles) {
+    const int least = std::max(1, (max_tiles + G - 1) / G);
+    const int many = std::max(least, max_tiles >= kMidFrom && max_tiles <= kMidTo ? kMidItemTiles : kItemTiles);
+    int active = 0;
+    for (int t : tiles) active += t > 0;
+    if (static_cast<int64_t>(active) * n_lb > G) return many;
+    auto rounds = [&](int c, int* longest) {
+        int64_t items = 0;
+        *longest = 0;
+        for (int t : tiles) {
+            if (t == 0) continue;
+            const int m = (t + c - 1) / c;
+            items += m;
+            *longest = std::max(*longest, (t + m - 1) / m);
+        }
+        return (items * n_lb + G - 1) / G;
+    };
+    int best = many, longest;
+    if (rounds(kItemTiles, &longest) > kFewRounds) return best;
+    float best_cost = 0.f;
+    for (int c = least; c <= kMaxItemTiles; ++c) {
+        const float r = static_cast<float>(rounds(c, &longest));
+        const float cost = r * (static_cast<float>(longest) + 2.f) + 0.25f * static_cast<float>(longest);
+        if (best_cost == 0.f || cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
+// The items of one launch of the two-pass kernel: unit (lb, s), of tiles[s] key tiles, is
+// split into m = ceil(tiles / c) items of balanced length, unit after unit (head batch major), c from
+// item_tiles; `units` ends with an entry holding the total.
 void plan_items(const std::vector<int>& tiles, int n_lb, int G, std::vector<LaunchUnit>& units) {
     units.clear();
     int max_tiles = 0;
     for (int t : tiles) max_tiles = std::max(max_tiles, t);
-    const int c = std::max(kItemTiles, (max_tiles + G - 1) / G);
+    const int c = item_tiles(tiles, n_lb, G, max_tiles);
     int item = 0;
     for (int lb = 0; lb < n_lb; ++lb)
         for (int s = 0; s < static_cast<int>(tiles.size()); ++s) {
@@ -693,9 +740,11 @@ ckv_status enqueue_layers(const std::vector<LayerJob>& jobs, const ckv_batch* b,
 // Whether the single-layer scoring runs on the TMEM-resident kernel (score_resident.cu); the
 // two-pass reload kernel otherwise.  CKV_ERR_UNSUPPORTED when the caller asked for the resident
 // kernel and a sequence does not fit it.
-// By itself it takes N = 32, and N = 64 while the call is small (up to four key tiles and half a unit
-// per CTA), so that one round of short items does it: one layer of 2048 / 8192 tokens 12.8 / 22.7 us
-// against 21.0 / 26.6 on the two-pass kernel, at 16384 (seven tiles per CTA) 41.5 against 26.6.
+// By itself it takes a small call (up to two key tiles per CTA, at N = 64 with at most half a unit: one
+// round of short items), and at N = 32 also a large one (more than four key tiles per CTA).  One layer, resident /
+// two-pass, us a call with the selection: N = 64, 2048 tokens 24.7 / 25.9, 4096 28.9 / 28.9, 6000 34.9 /
+// 31.0, 8192 37.1 / 33.1, 16384 64.1 / 41.9, two head batches of 2048 28.7 / 30.7, of 4096 37.0 / 35.0;
+// N = 32, 2048 22.8 / 24.6, 6000 30.9 / 28.9, 8192 33.0 / 28.9, 16384 35.0 / 37.0, 131072 98.4 / 114.6.
 ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int ctas, bool* resident) {
     int max_tiles = 0;
     int64_t tiles = 0, units = 0;
@@ -707,7 +756,8 @@ ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int 
         tiles += static_cast<int64_t>(t) * pl.nb;
         units += pl.nb;
     }
-    const bool small = tiles <= 4ll * ctas && 2 * units <= ctas;
+    const bool automatic = pl.n_cols == 32 ? tiles <= 2ll * ctas || tiles > 4ll * ctas
+                                           : tiles <= 2ll * ctas && 2 * units <= ctas;
     const int c_res = 512 / pl.n_cols;
     const bool fits = static_cast<long long>(max_tiles) <= static_cast<long long>(c_res) * ctas;
     if (pl.score_path == CKV_SCORE_RESIDENT && !fits)
@@ -716,7 +766,7 @@ ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int 
                     "on at least %d CTAs (%d available)", max_tiles, c_res,
                     (max_tiles + c_res - 1) / c_res, ctas);
     *resident = fits && (pl.score_path == CKV_SCORE_RESIDENT ||
-                         (pl.score_path == CKV_SCORE_AUTO && (pl.n_cols == 32 || small)));
+                         (pl.score_path == CKV_SCORE_AUTO && automatic));
     return CKV_OK;
 }
 

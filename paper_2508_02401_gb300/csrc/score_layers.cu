@@ -71,8 +71,8 @@ constexpr int kQBufs = 2;     // query-row buffers: pass 1 runs up to one item a
 // tiles evict-first in pass 1: their re-reads come after most of L2 has turned over.
 constexpr int kLongUnitKeys = 65536;
 constexpr int kItemRing = 8;  // item indices posted by the producer (more than any role's lag)
-// Largest |log2| of an item's column maximum: an item's sum is then below 2^1000 (at most
-// 2^10 keys), and the sum of up to 2^20 items stays below fp64's 2^1024.
+// Largest |log2| of an item's column maximum: a unit has at most 2^22 keys, so its sum stays below
+// 2^1012, within fp64's 2^1024.
 constexpr double kMaxLog2 = 990.0;
 
 template <int N>

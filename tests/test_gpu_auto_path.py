@@ -1,5 +1,5 @@
-"""The automatic choice of the one-layer scoring kernel at N = 64: small calls take the TMEM-resident
-kernel, larger ones the two-pass kernel.  Around the limits of the rule (key tiles and units per CTA),
+"""The automatic choice of the one-layer scoring kernel: small calls take the TMEM-resident kernel, as
+do large ones at N = 32, the others the two-pass kernel.  Around the limits of the rule (key tiles and units per CTA),
 with both layouts of K, the scores agree with the two-pass kernel's and the layer with the oracle."""
 import numpy as np
 import pytest
@@ -12,9 +12,9 @@ from tests import gpu_util as gu
 
 pytestmark = pytest.mark.gpu
 
-# 8 groups: 608 tiles of 152 CTAs is 76 per unit (9728 tokens); 76 units is 9 sequences
-CASES = [((130,), 2), ((2048,), 2), ((9728,), 2), ((9729,), 2), ((700,) * 9, 2), ((500,) * 10, 2),
-         ((4000, 33, 1, 3000), 2), ((1500,), 4)]
+# 8 groups: two tiles for each of 152 CTAs are 38 per unit (4864 tokens), four 76; 76 units are 9 sequences
+CASES = [((130,), 2), ((2048,), 2), ((4864,), 2), ((4865,), 2), ((500,) * 9, 2), ((400,) * 10, 2),
+         ((4000, 33, 1, 3000), 2), ((1500,), 4), ((4864,), 1), ((4865,), 1), ((9728,), 1), ((9729,), 1)]
 
 
 @pytest.mark.parametrize("interleaved", [False, True])

@@ -82,8 +82,8 @@ typedef enum ckv_scope {
 
 /* Which scoring kernel runs the two passes over the keys (same scores either way). */
 typedef enum ckv_score_path {
-    CKV_SCORE_AUTO = 0,     /* resident when it fits and the call is small, or large with N = 32
-                               (see below), otherwise reload */
+    CKV_SCORE_AUTO = 0,     /* resident when it fits and N = 32 (see below) or the call is small,
+                               otherwise reload */
     CKV_SCORE_RESIDENT = 1, /* each key tile is read and multiplied once; pass 1 keeps its
                                exponentials in tensor memory and pass 2 rescales them.  Needs
                                every sequence's key tiles to fit one round of work items of at

@@ -740,11 +740,12 @@ ckv_status enqueue_layers(const std::vector<LayerJob>& jobs, const ckv_batch* b,
 // Whether the single-layer scoring runs on the TMEM-resident kernel (score_resident.cu); the
 // two-pass reload kernel otherwise.  CKV_ERR_UNSUPPORTED when the caller asked for the resident
 // kernel and a sequence does not fit it.
-// By itself it takes a small call (up to two key tiles per CTA, at N = 64 with at most half a unit: one
-// round of short items), and at N = 32 also a large one (more than four key tiles per CTA).  One layer, resident /
+// By itself it takes N = 32, and N = 64 while the call is small (up to two key tiles and half a unit per
+// CTA: one round of short items).  One layer, resident /
 // two-pass, us a call with the selection: N = 64, 2048 tokens 24.7 / 25.9, 4096 28.9 / 28.9, 6000 34.9 /
 // 31.0, 8192 37.1 / 33.1, 16384 64.1 / 41.9, two head batches of 2048 28.7 / 30.7, of 4096 37.0 / 35.0;
-// N = 32, 2048 22.8 / 24.6, 6000 30.9 / 28.9, 8192 33.0 / 28.9, 16384 35.0 / 37.0, 131072 98.4 / 114.6.
+// N = 32, 2048 22.8 / 24.6, 8192 33.0 / 28.9, 16384 35.0 / 37.0, 131072 98.4 / 114.6 (around 8192 the
+// resident kernel stays, as its error against 64 bits is a tenth smaller: 2.2e-7 against 2.5e-7).
 ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int ctas, bool* resident) {
     int max_tiles = 0;
     int64_t tiles = 0, units = 0;
@@ -756,8 +757,7 @@ ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int 
         tiles += static_cast<int64_t>(t) * pl.nb;
         units += pl.nb;
     }
-    const bool automatic = pl.n_cols == 32 ? tiles <= 2ll * ctas || tiles > 4ll * ctas
-                                           : tiles <= 2ll * ctas && 2 * units <= ctas;
+    const bool automatic = pl.n_cols == 32 || (tiles <= 2ll * ctas && 2 * units <= ctas);
     const int c_res = 512 / pl.n_cols;
     const bool fits = static_cast<long long>(max_tiles) <= static_cast<long long>(c_res) * ctas;
     if (pl.score_path == CKV_SCORE_RESIDENT && !fits)

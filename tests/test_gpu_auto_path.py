@@ -1,5 +1,5 @@
 """The automatic choice of the one-layer scoring kernel: small calls take the TMEM-resident kernel, as
-do large ones at N = 32, the others the two-pass kernel.  Around the limits of the rule (key tiles and units per CTA),
+do all at N = 32, the others the two-pass kernel.  Around the limits of the rule (key tiles and units per CTA),
 with both layouts of K, the scores agree with the two-pass kernel's and the layer with the oracle."""
 import numpy as np
 import pytest

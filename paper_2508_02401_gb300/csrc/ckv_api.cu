@@ -573,13 +573,15 @@ struct LayerJob {
 // tail of about a quarter of an item; the length that makes this least is taken, so that the items
 // fill whole rounds.  14 tiles -> this rule, us a call: one layer of 8192 / 16384 / 32768 / 65536 tokens
 // 26.7 -> 18.6 / 26.7 -> 20.8 / 28.6 (14 tiles) / 49.7 -> 47.1; of 8192 tokens 2 layers 28.9 -> 24.6,
-// 4 layers 37.1 -> 30.8, 8 layers 52.7 -> 49.0; with the lse given 43.0 -> 41.2, -, 62.7 -> 59.8 (with
-// the selection).  More units than CTAs, or more than six rounds, even out by themselves.
+// 4 layers 37.1 -> 30.8, 8 layers 52.7 -> 49.0.  More units than CTAs, or more than six rounds, even out
+// by themselves.  With the lse given an item costs little more than its tiles (no exchange), so such
+// a launch takes items of four: with the selection, 2 / 8 layers of 8192 tokens 43.2 -> 41.3 / 62.7 ->
+// 58.8 us a call, 4 of 32768 96.8 -> 95.2 (8 tiles: 41.5, 59.6, 95.1; 2 tiles: 43.3, 65.4, 107.1).
 constexpr int kItemTiles = 14;
 constexpr int kMidItemTiles = 12;                      // where the longest sequence has
 constexpr int kMidFrom = 160, kMidTo = 512;            // this many tiles
-constexpr int kFewRounds = 6, kMaxItemTiles = 16;
-int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles) {
+constexpr int kFewRounds = 6, kMaxItemTiles = 16, kLseItemTiles = 4;
+int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles, bool given_lse) {
     const int least = std::max(1, (max_tiles + G - 1) / G);
     const int many = std::max(least, max_tiles >= kMidFrom && max_tiles <= kMidTo ? kMidItemTiles : kItemTiles);
     int active = 0;
@@ -598,6 +600,7 @@ int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles) {
     };
     int best = many, longest;
     if (rounds(kItemTiles, &longest) > kFewRounds) return best;
+    if (given_lse) return std::max(least, kLseItemTiles);
     float best_cost = 0.f;
     for (int c = least; c <= kMaxItemTiles; ++c) {
         const float r = static_cast<float>(rounds(c, &longest));
@@ -613,11 +616,11 @@ int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles) {
 // The items of one launch of the two-pass kernel: unit (lb, s), of tiles[s] key tiles, is
 // split into m = ceil(tiles / c) items of balanced length, unit after unit (head batch major), c from
 // item_tiles; `units` ends with an entry holding the total.
-void plan_items(const std::vector<int>& tiles, int n_lb, int G, std::vector<LaunchUnit>& units) {
+void plan_items(const std::vector<int>& tiles, int n_lb, int G, bool given_lse, std::vector<LaunchUnit>& units) {
     units.clear();
     int max_tiles = 0;
     for (int t : tiles) max_tiles = std::max(max_tiles, t);
-    const int c = item_tiles(tiles, n_lb, G, max_tiles);
+    const int c = item_tiles(tiles, n_lb, G, max_tiles, given_lse);
     int item = 0;
     for (int lb = 0; lb < n_lb; ++lb)
         for (int s = 0; s < static_cast<int>(tiles.size()); ++s) {
@@ -714,7 +717,7 @@ ckv_status enqueue_layers(const std::vector<LayerJob>& jobs, const ckv_batch* b,
                 for (int h : J.pl->sel_heads) L.sel_heads.push_back(static_cast<int16_t>(h));
                 L.layers.push_back(ly);
             }
-            plan_items(tiles, nb, ctas, L.units);
+            plan_items(tiles, nb, ctas, jobs[j0].lse != nullptr, L.units);
             L.seq0 = s0;
             L.S_all = S;
             L.cu_seqlens_dev = b->cu_seqlens_dev;

@@ -297,7 +297,7 @@ __device__ __forceinline__ bool item_partials(float (&m)[kCols], float (&s)[kCol
             const float2 x = red[q * 32 + wtid];
             S += x.y * ex2_approx(x.x - M);
         }
-        if (!mbar_wait(pub_empty, pub_phase ^ 1, abort, lim)) return false;
+        if (!__all_sync(0xffffffffu, mbar_wait(pub_empty, pub_phase ^ 1, abort, lim))) return false;
         out[wtid] = make_float2(M, S);
         mbar_arrive(pub_full);
     }

@@ -485,11 +485,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 int gi = -1;
-                if (!wait_item<kItemRing>(item_full, items, it, &gi, abort, lim)) {
-                    ok = false;
-                    break;
-                }
-                if (gi < 0) break;
+                ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
+                if (!ok || gi < 0) break;
                 const Item I = get_item(p, gi);
                 const int n = I.ntiles;
                 const int L = I.len, P = L - p.w;
@@ -505,10 +502,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                 }
                 for (int jt = 0; jt < n; ++jt, ++a_it) {
                     const int acc = a_it % kAcc;
-                    if (!mbar_wait(&a_full[acc], (a_it / kAcc) & 1, abort, lim)) {
-                        ok = false;
-                        break;
-                    }
+                    // (the warp decides as one: the tcgen05.ld below is warp-collective)
+                    ok = __all_sync(0xffffffffu, mbar_wait(&a_full[acc], (a_it / kAcc) & 1, abort, lim));
+                    if (!ok) break;
                     tc_fence_after_sync();
                     const int t = I.tile0 + jt;
                     const int j = t * kTileKeys + eq * 32 + lane;  // sequence-local key
@@ -591,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
                     }
                 }
             }
-            if (!group_sync(group, gphase, abort, lim) || *abort) {
+            if (!group_sync(group, gphase, abort, lim) || __any_sync(0xffffffffu, *abort != 0)) {
                 ok = false;
                 break;
             }
@@ -615,10 +611,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
             // ---------------------------------------------------- the item's tiles
             for (int jt = 0; jt < n; ++jt, ++b_it) {
                 const int acc = b_it % kAcc;
-                if (!mbar_wait(&b_full[acc], (b_it / kAcc) & 1, abort, lim)) {
-                    ok = false;
-                    break;
-                }
+                ok = __all_sync(0xffffffffu, mbar_wait(&b_full[acc], (b_it / kAcc) & 1, abort, lim));
+                if (!ok) break;
                 tc_fence_after_sync();
                 const int t = tile0 + jt;
                 const int j = t * kTileKeys + eq * 32 + lane;

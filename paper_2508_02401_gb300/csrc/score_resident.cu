@@ -431,10 +431,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_resident_kernel(const __gri
 #pragma unroll
                 for (int i = 0; i < kCols; ++i) m[i] = -nm[i];
                 // the warp's references for pass 2, once it has read those of the item two back
-                if (!mbar_wait(&m_empty[a_item & 1], ((a_item >> 1) & 1) ^ 1, abort, lim)) {
-                    ok = false;
-                    break;
-                }
+                ok = __all_sync(0xffffffffu, mbar_wait(&m_empty[a_item & 1], ((a_item >> 1) & 1) ^ 1, abort, lim));
+                if (!ok) break;
                 if (lane == 0) {
                     float4* dst = reinterpret_cast<float4*>(&ref_s[a_item & 1][eq][col0]);
 #pragma unroll

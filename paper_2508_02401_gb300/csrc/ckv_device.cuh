@@ -74,6 +74,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                  : "memory");
 }
 
+// Suspends until the phase with the given parity completes or a time limit of the hardware's.
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -99,31 +100,20 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// try_wait with a suspend-time hint: the thread sleeps in the barrier unit until the phase
-// completes or about `ns` nanoseconds have passed, so a waiting warp takes no issue slots.
-__device__ __forceinline__ bool mbar_try_wait_for(uint64_t* bar, uint32_t parity, uint32_t ns) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
-        : "memory");
-    return ok != 0;
-}
-
 // Waits for the phase with the given parity to complete.  Gives up (returns false) after
 // `limit` cycles or once *abort is set by another thread of the block; both are checked each
-// time a suspended try_wait (at most ~1 us) returns without the phase.
-constexpr uint32_t kSuspendNs = 1000;
+// time a try_wait returns without the phase.  A try_wait suspends the thread in the barrier unit, so
+// that a waiting warp takes no issue slots, until the phase completes or about 7800 cycles (3.8 us)
+// have passed; a suspend-time hint of 0.1 to 20 us changes nothing in that.  Under a limit of the
+// same order the thread therefore polls: 1 us then means 1 us.
+constexpr long long kPollCycles = 200000;  // limits up to this (about 100 us) are polled
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           long long limit = kWaitTimeoutCycles) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
 #pragma unroll 1
     for (;;) {
-        if (mbar_try_wait_for(bar, parity, kSuspendNs)) return true;
+        if (limit > kPollCycles ? mbar_try_wait(bar, parity) : mbar_test(bar, parity)) return true;
         if (*abort || clock64() - t0 > limit) return false;
     }
 }

@@ -1292,6 +1292,7 @@ struct SelectLayersParams {
     int unit_jobs[kSelMaxLayers];    // jobs of each unit of a long sequence
     int long_seq[kSelMaxLongSeqs];   // the sequences of more than `own` tokens (where there are jobs)
     int key_stride;                  // select_key_stride(T, S)
+    long long wait_cycles;           // limit of a bounded wait (ckv_set_wait_limit_us)
 };
 
 __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __grid_constant__ SelectLayersParams P) {
@@ -1432,12 +1433,14 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
                 }
                 if (tma) {  // this chunk's loads have landed (a bounded wait)
                     const int b = bi;
-                    const bool ok = mbar_wait(&tbar[b], (tph >> b) & 1u, &s_abort);
+                    const bool ok = mbar_wait(&tbar[b], (tph >> b) & 1u, &s_abort, P.wait_cycles);
                     tph ^= 1u << b;
                     if (__syncthreads_or(ok ? 0 : 1)) {
-                        // give up: report, let the loads still in flight land, leave
+                        // give up: report, release the unit's jobs, let the loads still in flight
+                        // land, leave
                         if (tid == 0) {
                             record_error(p.status, kDevTimeout, 250);
+                            if (prev >= 0) st_release(unit_done + prev, 2);
                             volatile int never = 0;
                             mbar_wait(&tbar[b], ((tph >> b) & 1u) ^ 1u, &never);
                             if (more && nb == 2) mbar_wait(&tbar[b ^ 1], (tph >> (b ^ 1)) & 1u, &never);
@@ -1972,6 +1975,7 @@ cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, 
         P.units_per_layer = Ls[l0].S * Ls[l0].n_vec * P.copies;
         P.key_stride = select_key_stride(Ls[l0].T, Ls[l0].S);
         P.next_unit = next_unit;
+        P.wait_cycles = wait_limit_cycles();
         const int units = nl * P.units_per_layer;
         if (units == 0) continue;
         // Row-copy jobs, unless so many sequences are long that the units themselves spread the rows.

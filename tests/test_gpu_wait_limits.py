@@ -1,6 +1,8 @@
 """Bounded waits that run out, kernel by kernel: the call returns, the status word reports it, and the
 same call with the default limit is clean and matches the oracle.  The limit is shortened with
 ckv_set_wait_limit_us; no flag, barrier or check is removed, every wait still ends."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -103,3 +105,50 @@ def test_a_wait_that_is_suspended_gives_up():
     assert g["status"][0] == 2, g["status"]
     g = gu.run_gpu(wl, 0, li, cfg=cfg)
     gu.check_layer(wl, 0, li, g, gu.run_oracle(wl, 0, li, want_kv=False))
+
+
+def _fill(ios):
+    for io in ios:
+        io.idx.fill_(-7)
+
+
+def _check_clean(wl, cfg, batch, layers):
+    """The call with the default limit: status clean, positions and rows as the oracle's."""
+    ios = [io for io, _ in layers]
+    for io in ios:
+        io.pooled_out = torch.zeros((cfg.num_vectors, batch.total_tokens), dtype=torch.float32, device="cuda")
+    ws = ckv.new_layers_workspace(cfg, ios, batch)
+    ckv.ckv_compress_layers_lse(cfg, ios, batch, ws)
+    assert ckv.ckv_read_device_status(ws) == (0, 0)
+    for l, (io, li) in enumerate(layers):
+        g = dict(cfg=cfg, cu_keep=ckv.ckv_keep_lengths(cfg, l, batch)[0], pooled=io.pooled_out.cpu().numpy(),
+                 idx=io.idx.cpu().numpy(), cu_keep_dev=io.cu_keep_dev.cpu().numpy(),
+                 k_out=gu.to_host(io.k_out), v_out=gu.to_host(io.v_out))
+        gu.check_layer(wl, l, li, g, gu.run_oracle(wl, l, li, want_kv=False))
+
+
+def test_a_selection_that_gives_up_releases_its_row_copy_jobs():
+    """Four score rows a selection are staged in one buffer, so that every chunk waits for its loads, longer
+    than 1 us: the units of the long sequence give up.  Those of the short ones, kept whole, stage
+    nothing; their CTAs go on to the long units' row-copy jobs and must not wait for them."""
+    wl = cs.Workload(name="limits_stage", num_layers=1, num_q_heads=8, num_kv_heads=2, seqlens=(60000,) + (1000,) * 12,
+                     window=16, heads_per_group=4, budget_mean=1100, budget_uniform=True, seed=41)
+    cfg, batch = ckv.Config.from_workload(wl), ckv.Batch(wl.cu_seqlens())
+    layers = _layers(wl, cfg, batch, lse=True)
+    ios = [io for io, _ in layers]
+    ws = ckv.new_layers_workspace(cfg, ios, batch)
+    ckv.ckv_compress_layers_lse(cfg, ios, batch, ws)  # loads the kernels
+    assert ckv.ckv_read_device_status(ws) == (0, 0)
+    _fill(ios)
+    ckv.ckv_set_wait_limit_us(1)
+    try:
+        t0 = time.perf_counter()
+        ckv.ckv_compress_layers_lse(cfg, ios, batch, ws)
+        assert ckv.ckv_read_device_status(ws)[0] == 2
+        took = time.perf_counter() - t0
+    finally:
+        ckv.ckv_set_wait_limit_us(0)
+    idx = ios[0].idx.cpu().numpy()
+    assert np.all(idx[:, :1100] == -7) and np.all(idx[:, 1100:] >= 0)  # who gave up, and who did not
+    assert took < 1.0, took  # a job that waits for a unit that gave up waits about 2 s
+    _check_clean(wl, cfg, batch, layers)

@@ -1713,7 +1713,7 @@ __global__ void __launch_bounds__(kLsThreads, 1) select_layers_kernel(const __gr
             const int* flag = unit_done + li * P.units_per_layer + lu;
             const long long t0 = clock64();
             int f;
-            while ((f = ld_acquire_gpu(flag)) == 0 && clock64() - t0 <= kWaitTimeoutCycles) __nanosleep(64);
+            while ((f = ld_acquire_gpu(flag)) == 0 && clock64() - t0 <= P.wait_cycles) __nanosleep(64);
             if (f == 0) record_error(p.status, kDevTimeout, 251);
             s_cnt = f;
         }

@@ -152,3 +152,22 @@ def test_a_selection_that_gives_up_releases_its_row_copy_jobs():
     assert np.all(idx[:, :1100] == -7) and np.all(idx[:, 1100:] >= 0)  # who gave up, and who did not
     assert took < 1.0, took  # a job that waits for a unit that gave up waits about 2 s
     _check_clean(wl, cfg, batch, layers)
+
+
+def test_a_row_copy_job_whose_unit_takes_longer_than_the_limit_is_reported():
+    """The units of the short sequences, kept whole, end within some 25 us; their CTAs go on to the jobs of
+    the long sequence's units, which take about 100 us: a limit of 30 us runs out there (detail 251) and
+    nowhere before, as the given-lse scoring's waits take a few microseconds."""
+    wl = cs.Workload(name="limits_jobs", num_layers=1, num_q_heads=8, num_kv_heads=2, seqlens=(131072,) + (600,) * 12,
+                     window=32, heads_per_group=2, budget_mean=1100, budget_uniform=True, seed=43)
+    cfg, batch = ckv.Config.from_workload(wl), ckv.Batch(wl.cu_seqlens())
+    layers = _layers(wl, cfg, batch, lse=True)
+    ios = [io for io, _ in layers]
+    ws = ckv.new_layers_workspace(cfg, ios, batch)
+    ckv.ckv_set_wait_limit_us(30)
+    try:
+        ckv.ckv_compress_layers_lse(cfg, ios, batch, ws)
+        assert ckv.ckv_read_device_status(ws) == (2, 251)
+    finally:
+        ckv.ckv_set_wait_limit_us(0)
+    _check_clean(wl, cfg, batch, layers)

@@ -564,7 +564,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_layers_kernel(const __grid_
             ok = __all_sync(0xffffffffu, wait_item<kItemRing>(item_full, items, it, &gi, abort, lim));
             if (!ok || gi < 0) break;
             // pass 2 reads an item's ring entry last: once each of its warps has, the producer
-            // may post another item there
+            // may post another item there (a vote does not order the lanes' reads before the arrival)
+            __syncwarp();
             if (lane == 0) mbar_arrive(&item_free[it % kItemRing]);
             const Item I = get_item(p, gi);
             const int n = I.ntiles, tile0 = I.tile0;

@@ -532,6 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_lse_layers_kernel(const __g
             for (int it = 0; ok; ++it) {
                 int gi = -1;
                 ok = __all_sync(0xffffffffu, wait_item<kLseItemRing>(item_full, items, it, &gi, abort, lim));
+                __syncwarp();  // every lane has read the entry (a vote alone does not order the reads)
                 if (leader) mbar_arrive(&item_free[it % kLseItemRing]);
                 if (!ok || gi < 0) break;
                 const int n = get_item(p, gi).ntiles;
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_lse_layers_kernel(const __g
         for (int it = 0; ok; ++it) {
             int gi = -1;
             ok = __all_sync(0xffffffffu, wait_item<kLseItemRing>(item_full, items, it, &gi, abort, lim));
+            __syncwarp();  // every lane has read the entry
             if (lane == 0) mbar_arrive(&item_free[it % kLseItemRing]);
             if (!ok) break;
             if (gi < 0) break;

@@ -760,7 +760,9 @@ ckv_status resident_choice(const Plan& pl, const ckv_batch* b, int skip_le, int 
         tiles += static_cast<int64_t>(t) * pl.nb;
         units += pl.nb;
     }
-    const bool automatic = pl.n_cols == 32 || (tiles <= 2ll * ctas && 2 * units <= ctas);
+    // (the resident kernel's tables take 65535 sequences; the two-pass kernel any number of them)
+    const bool automatic = pl.n_cols == 32 ||
+                           (b->num_seqs <= 65535 && tiles <= 2ll * ctas && 2 * units <= ctas);
     const int c_res = 512 / pl.n_cols;
     const bool fits = static_cast<long long>(max_tiles) <= static_cast<long long>(c_res) * ctas;
     if (pl.score_path == CKV_SCORE_RESIDENT && !fits)

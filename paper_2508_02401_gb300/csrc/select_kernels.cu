@@ -1860,11 +1860,7 @@ cudaError_t launch_gather(const GatherLaunch& L, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-// The selection of several layers in one launch (select_layers_kernel); Ls[i] as for
-// launch_select with from_scores = 1, and keys[i] a [H_kv, select_key_stride(T, S)] scratch of
-// 8-byte (key, position) slots per layer.  One launch per
-// kSelMaxLayers layers; `next_unit` (kSelMaxLayers-aligned count of ints) is the work counter
-// of each launch and is cleared first.
+// Ints of work counters (units, row-copy jobs) and done flags (one per unit) of a launch.
 int select_counters(int units_per_layer) { return 2 + kSelMaxLayers * units_per_layer; }
 
 int select_key_stride(int T, int S) { return (T + 4 * S + 3) & ~3; }
@@ -1882,10 +1878,11 @@ int select_key_stride(int T, int S) { return (T + 4 * S + 3) & ~3; }
 //   32 layers of eight prompts of 2048:                8: 267    461 / 350 / 298 /  -
 //   32 layers of one prompt of 32768, budget 1024:     2: 343    351 /  -  / 392 / 502
 //   8 layers of one prompt of 131072, budget 1024:     1: 441     -  / 465 / 516 / 617
-int heads_per_unit(const SelectLaunch* Ls, const int* order, int nl, int grid) {
-    const int Hkv = Ls[order[0]].Hkv, S = Ls[order[0]].S;
+// budgets and score_rows are those of the launch's nl layers, the largest budgets first (a budget of 0
+// where no rows are copied).
+int select_heads_per_unit(const int* budgets, const int* score_rows, int nl, int S, int T, int Hkv, int grid) {
     if (S <= 0) return 1;
-    const int len = Ls[order[0]].T / S;
+    const int len = T / S;
     const float chunks = static_cast<float>((len + kLsChunk - 1) / kLsChunk);
     int best = 1;
     float best_us = 0.f;
@@ -1893,9 +1890,8 @@ int heads_per_unit(const SelectLaunch* Ls, const int* order, int nl, int grid) {
         const long long per = static_cast<long long>(S) * ((Hkv + h - 1) / h);  // units of a layer
         float t[kSelMaxLayers], us = 0.f;
         for (int i = 0; i < nl; ++i) {
-            const SelectLaunch& L = Ls[order[i]];
-            const int rows = L.k ? std::min(std::min(L.budget, len), kSelectOwnRows) : 0;
-            t[i] = 16.f + chunks * (2.f + 0.5f * static_cast<float>(L.group_first[1])) +
+            const int rows = std::min(std::min(budgets[i], len), kSelectOwnRows);
+            t[i] = 16.f + chunks * (2.f + 0.5f * static_cast<float>(score_rows[i])) +
                    0.017f * static_cast<float>(std::min(h, Hkv)) * static_cast<float>(rows);
             us += t[i] * static_cast<float>(per) / static_cast<float>(grid);
         }
@@ -1910,6 +1906,11 @@ int heads_per_unit(const SelectLaunch* Ls, const int* order, int nl, int grid) {
     return best;
 }
 
+// The selection of several layers in one launch (select_layers_kernel); Ls[i] as for
+// launch_select with from_scores = 1, and keys[i] a [H_kv, select_key_stride(T, S)] scratch of
+// 8-byte (key, position) slots per layer.  One launch per kSelMaxLayers layers; `next_unit` holds
+// select_counters(units per layer) ints, of which each launch clears the two counters, and the flags
+// too where it has row-copy jobs.
 cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, int n_layers,
                                  int* next_unit, int grid, cudaStream_t stream) {
     static SelectLayersParams P;  // ~25 KB; calls are serialised by `mu`
@@ -1969,7 +1970,12 @@ cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, 
         P.n_layers = nl;
         P.copies = P.heads = 1;
         if (Ls[l0].n_vec == 1) {
-            P.heads = heads_per_unit(Ls, order, nl, grid);
+            int budgets[kSelMaxLayers], score_rows[kSelMaxLayers];
+            for (int i = 0; i < nl; ++i) {
+                budgets[i] = Ls[order[i]].k ? Ls[order[i]].budget : 0;
+                score_rows[i] = Ls[order[i]].group_first[1];
+            }
+            P.heads = select_heads_per_unit(budgets, score_rows, nl, Ls[l0].S, Ls[l0].T, Ls[l0].Hkv, grid);
             P.copies = (Ls[l0].Hkv + P.heads - 1) / P.heads;
         }
         P.units_per_layer = Ls[l0].S * Ls[l0].n_vec * P.copies;
@@ -2010,3 +2016,11 @@ cudaError_t launch_select_layers(const SelectLaunch* Ls, uint32_t* const* keys, 
 }
 
 }  // namespace ckv
+
+// The rule of the KV heads per unit, for the tests (host only; not part of the ABI).
+extern "C" __attribute__((visibility("default"))) int32_t ckv_internal_select_heads_per_unit(
+    const int32_t* budgets, const int32_t* score_rows, int32_t n_layers, int32_t S, int32_t T, int32_t Hkv,
+    int32_t ctas) {
+    if (n_layers < 1 || n_layers > ckv::kSelMaxLayers) return -1;
+    return ckv::select_heads_per_unit(budgets, score_rows, n_layers, S, T, Hkv, ctas);
+}

@@ -1,0 +1,24 @@
+"""The multi-layer selection's choice of KV heads per unit (one selection per layer), on the host."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import ckv_synth as cs
+import paper_2508_02401_gb300 as ckv
+from paper_2508_02401_gb300 import build as ckv_build
+
+
+@pytest.mark.parametrize("layers,seqs,length,budget,kv_heads,want", [
+    (8, 1, 8192, 256, 8, 1), (32, 1, 8192, 256, 8, 2), (32, 4, 8192, 256, 8, 4), (32, 8, 2048, 256, 8, 8),
+    (32, 1, 32768, 1024, 8, 2), (8, 1, 131072, 1024, 8, 1), (8, 8, 300, 100, 3, 2), (8, 12, 300, 100, 3, 3),
+    (8, 8, 300, 100, 5, 4), (32, 1, 600, 100, 1, 1)])
+def test_heads_per_unit(layers, seqs, length, budget, kv_heads, want):
+    """152 CTAs, four score rows, layer-adaptive budgets; the first six are shapes that the rule was fitted to."""
+    ckv_build.build()
+    wl = cs.Workload(name="rule", num_layers=layers, num_q_heads=4 * kv_heads, num_kv_heads=kv_heads, window=32,
+                     heads_per_group=1, budget_mean=budget, seqlens=(length,) * seqs, seed=1)
+    b, r = np.sort(wl.budgets().astype(np.int32))[::-1].copy(), np.full(layers, 4, np.int32)
+    got = ckv.load().ckv_internal_select_heads_per_unit(
+        b.ctypes.data_as(ctypes.c_void_p), r.ctypes.data_as(ctypes.c_void_p), layers, seqs, seqs * length, kv_heads, 152)
+    assert got == want

@@ -9,6 +9,7 @@ import oracle
 import paper_2508_02401_gb300 as ckv
 from tests import gpu_util as gu
 from tests import test_gpu_layers as layers
+from tests import test_gpu_wait_limits as limits
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +32,34 @@ def test_item_lengths(case, max_ctas):
     res = layers._run_layers(wl, cfg, lis, with_scores=True)
     for l, li in enumerate(lis):
         gu.check_layer(wl, l, li, res[l], gu.run_oracle(wl, l, li, want_kv=False))
+
+
+# The given-lse kernel's items: of four tiles in a launch of up to six rounds (of 14-tile items), of 12 or
+# 14 tiles in one of more rounds or of more units than CTAs; a unit has at most as many items as CTAs.
+# 8 units a layer on 8 CTAs: 84 tiles (10752 tokens) are six rounds, 85 are seven.
+LSE_CASES = [((129,), 1, 0), ((2433,), 2, 0), ((10752,), 1, 8), ((10753,), 1, 8), ((20480,), 1, 8), ((65537,), 1, 8),
+             ((8192, 100), 2, 0), ((900, 1, 3000), 1, 37), ((300,) * 20, 1, 0), ((2000,), 1, 1)]
+
+
+@pytest.mark.parametrize("case", range(len(LSE_CASES)))
+def test_given_lse_item_lengths(case):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    oracle.build()
+    lens, n, max_ctas = LSE_CASES[case]
+    kv_heads = 1 if max_ctas == 1 else 8
+    wl = cs.Workload(name="items_lse", num_layers=n, num_q_heads=2 * kv_heads, num_kv_heads=kv_heads, seqlens=lens,
+                     window=32, heads_per_group=2, budget_mean=64, pool_kernel=7, seed=34)
+    cfg, batch = ckv.Config.from_workload(wl, max_ctas=max_ctas), ckv.Batch(wl.cu_seqlens())
+    ios = limits._layers(wl, cfg, batch, lse=True)
+    out = []
+    for io, _ in ios:
+        out.append(gu.Guarded(tuple(io.scores.shape), torch.float32, float("nan")))
+        io.scores = out[-1].view
+    ws = ckv.new_layers_workspace(cfg, [io for io, _ in ios], batch)
+    ckv.ckv_score_windows_lse(cfg, [io for io, _ in ios], batch, ws)
+    assert ckv.ckv_read_device_status(ws) == (0, 0)
+    for l, (g, (_, li)) in enumerate(zip(out, ios)):
+        g.check()
+        o = gu.run_oracle(wl, l, li, want_kv=False)
+        gu.assert_close_rows(g.view.cpu().numpy(), o["scores"])

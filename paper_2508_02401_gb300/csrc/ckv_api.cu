@@ -558,8 +558,9 @@ struct LayerJob {
     int64_t lse_stride = 0;
 };
 
-// Key tiles per item of a launch over n_lb head batches of sequences of tiles[s] key tiles.  At least
-// ceil(max_tiles / G), so that a unit has at most G items (the kernel's progress argument).
+// Key tiles per item of a launch over n_lb head batches of sequences of tiles[s] key tiles; 0: each
+// sequence by its own length (long_item_tiles).  At least `least` = ceil(longest / G), so that a unit has
+// at most G items (the kernel's progress argument).
 //
 // A launch of many rounds of items: long enough that an item's fixed costs (taking it, loading its
 // query rows, publishing its sums, the unit's lse) are paid rarely, and short enough that the faster
@@ -567,6 +568,11 @@ struct LayerJob {
 // 12 / 13 / 14 / 16 tiles: 32 layers of 131072 tokens 1851 / 1878 / 1905 / 1814 / -; 16 of 65536
 // 447 / 428 / 434 / 445 / -; 32 of 32768 435 / 427 / 429 / 436 / 495; 28 ragged 830 / 828 / 837 / 841 / -;
 // 32 of 16384 230 / 228 / 228 / 227 / -; 32 of 8192 - / 130 / 130 / 129 / 143.
+// 12 tiles for a sequence of 160 to 512 of them: each CTA has up to two items between a tile's two reads,
+// 139 MB over the GPU with items of 14 against an L2 of 129 MB, 119 MB with 12 (DRAM traffic of 8
+// layers of 32768 tokens 1.20 -> 1.07 of K, of the ragged batch 1.23 -> 1.11).  Shorter sequences complete
+// sooner than that and lose by it (16 layers of six of 8192 tokens and one of 20481: 459 with 12 for
+// all, 452 with 14 for all), longer ones miss L2 either way.
 //
 // A launch of few rounds lasts its rounds times the longest item (a tile takes about 0.9 us from its
 // load to its score, the two passes hardly overlap), a fixed cost a round of about two tiles, and a
@@ -578,15 +584,14 @@ struct LayerJob {
 // a launch takes items of four: with the selection, 2 / 8 layers of 8192 tokens 43.2 -> 41.3 / 62.7 ->
 // 58.8 us a call, 4 of 32768 96.8 -> 95.2 (8 tiles: 41.5, 59.6, 95.1; 2 tiles: 43.3, 65.4, 107.1).
 constexpr int kItemTiles = 14;
-constexpr int kMidItemTiles = 12;                      // where the longest sequence has
-constexpr int kMidFrom = 160, kMidTo = 512;            // this many tiles
+constexpr int kMidItemTiles = 12;                      // for a sequence
+constexpr int kMidFrom = 160, kMidTo = 512;            // of this many tiles
 constexpr int kFewRounds = 6, kMaxItemTiles = 16, kLseItemTiles = 4;
-int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles, bool given_lse) {
-    const int least = std::max(1, (max_tiles + G - 1) / G);
-    const int many = std::max(least, max_tiles >= kMidFrom && max_tiles <= kMidTo ? kMidItemTiles : kItemTiles);
+int long_item_tiles(int t) { return t >= kMidFrom && t <= kMidTo ? kMidItemTiles : kItemTiles; }
+int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int least, bool given_lse) {
     int active = 0;
     for (int t : tiles) active += t > 0;
-    if (static_cast<int64_t>(active) * n_lb > G) return many;
+    if (static_cast<int64_t>(active) * n_lb > G) return 0;
     auto rounds = [&](int c, int* longest) {
         int64_t items = 0;
         *longest = 0;
@@ -598,7 +603,7 @@ int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int max_tiles, bo
         }
         return (items * n_lb + G - 1) / G;
     };
-    int best = many, longest;
+    int best = 0, longest;
     if (rounds(kItemTiles, &longest) > kFewRounds) return best;
     if (given_lse) return std::max(least, kLseItemTiles);
     float best_cost = 0.f;
@@ -620,12 +625,14 @@ void plan_items(const std::vector<int>& tiles, int n_lb, int G, bool given_lse, 
     units.clear();
     int max_tiles = 0;
     for (int t : tiles) max_tiles = std::max(max_tiles, t);
-    const int c = item_tiles(tiles, n_lb, G, max_tiles, given_lse);
+    const int least = std::max(1, (max_tiles + G - 1) / G);
+    const int all = item_tiles(tiles, n_lb, G, least, given_lse);
     int item = 0;
     for (int lb = 0; lb < n_lb; ++lb)
         for (int s = 0; s < static_cast<int>(tiles.size()); ++s) {
             const int t = tiles[s];
             if (t == 0) continue;
+            const int c = all > 0 ? all : std::max(least, long_item_tiles(t));
             units.push_back(LaunchUnit{static_cast<int16_t>(lb), static_cast<int16_t>(s), item});
             item += std::min(t, (t + c - 1) / c);
         }
@@ -1591,6 +1598,19 @@ ckv_status ckv_score_window_static(const ckv_config* cfg, int32_t layer, const c
         if (e != cudaSuccess) return cuda_fail(e, "copying the static status word");
     }
     return CKV_OK;
+}
+
+// The items per unit of a multi-layer launch, for the tests (host only; not part of the ABI): sequence s
+// of tiles[s] key tiles is cut into items[s] of them.
+__attribute__((visibility("default"))) int32_t ckv_internal_plan_items(
+    const int32_t* tiles, int32_t n_seqs, int32_t n_batches, int32_t ctas, int32_t given_lse, int32_t* items) {
+    const std::vector<int> t(tiles, tiles + n_seqs);
+    std::vector<LaunchUnit> units;
+    plan_items(t, n_batches, ctas, given_lse != 0, units);
+    for (int s = 0; s < n_seqs; ++s) items[s] = 0;
+    for (size_t u = 0; u + 1 < units.size(); ++u)
+        if (units[u].lb == 0) items[units[u].seq] = units[u + 1].item0 - units[u].item0;
+    return units.back().item0;
 }
 
 }  // extern "C"

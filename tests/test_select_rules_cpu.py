@@ -1,4 +1,5 @@
-"""The multi-layer selection's choice of KV heads per unit (one selection per layer), on the host."""
+"""The rules of the multi-layer calls, on the host: KV heads per unit of the selection (one selection per
+layer), items per unit of the scoring."""
 import ctypes
 
 import numpy as np
@@ -22,3 +23,25 @@ def test_heads_per_unit(layers, seqs, length, budget, kv_heads, want):
     got = ckv.load().ckv_internal_select_heads_per_unit(
         b.ctypes.data_as(ctypes.c_void_p), r.ctypes.data_as(ctypes.c_void_p), layers, seqs, seqs * length, kv_heads, 152)
     assert got == want
+
+
+def _items(tiles, batches, ctas=152, lse=False):
+    t, out = np.array(tiles, np.int32), np.zeros(len(tiles), np.int32)
+    total = ckv.load().ckv_internal_plan_items(
+        t.ctypes.data_as(ctypes.c_void_p), len(t), batches, ctas, int(lse), out.ctypes.data_as(ctypes.c_void_p))
+    assert total == batches * out.sum()
+    return out.tolist()
+
+
+@pytest.mark.parametrize("lse", [False, True])
+def test_long_launches_cut_each_sequence_by_its_own_length(lse):
+    """32 layers of 8 KV heads: a sequence's items are the same alone and beside any other, 12 tiles from 160
+    to 512 tiles and 14 otherwise, and never more than the CTAs."""
+    ckv_build.build()
+    tiles = [161, 64, 64, 1024, 512, 513, 159, 160, 1, 0]
+    want = [14, 5, 5, 74, 43, 37, 12, 14, 1, 0]
+    assert _items(tiles, 256, lse=lse) == want
+    for t, m in zip(tiles, want):
+        if t >= 64:
+            assert _items([t], 256, lse=lse) == [m]
+    assert _items([161, 20000], 128, ctas=8, lse=lse) == [1, 8]

@@ -580,13 +580,20 @@ struct LayerJob {
 // fill whole rounds.  14 tiles -> this rule, us a call: one layer of 8192 / 16384 / 32768 / 65536 tokens
 // 26.7 -> 18.6 / 26.7 -> 20.8 / 28.6 (14 tiles) / 49.7 -> 47.1; of 8192 tokens 2 layers 28.9 -> 24.6,
 // 4 layers 37.1 -> 30.8, 8 layers 52.7 -> 49.0.  More units than CTAs, or more than six rounds, even out
-// by themselves.  With the lse given an item costs little more than its tiles (no exchange), so such
-// a launch takes items of four: with the selection, 2 / 8 layers of 8192 tokens 43.2 -> 41.3 / 62.7 ->
-// 58.8 us a call, 4 of 32768 96.8 -> 95.2 (8 tiles: 41.5, 59.6, 95.1; 2 tiles: 43.3, 65.4, 107.1).
+// by themselves.
+//
+// With the lse given an item costs little more than its tiles (no exchange: about one, and no tail).
+// Up to two rounds of 14 tiles, the least rounds times (longest item + 1); up to six, where the
+// rounds begin to blur, items of four.  With the selection, us a call, 14 tiles / four throughout /
+// this rule: one layer of 2048 39.4 / 37.8 / 37.0, of 8192 44.4 / 40.7 / 40.8, of 16384 46.3 / 44.9 /
+// 44.5, of 32768 58.7 / 58.9 / 58.5 tokens; 2 of twice 4096 46.5 / 46.7 / 45.4, 3 of 20000 69.2 /
+// 69.5 / 69.8; beyond two rounds 8 of 8192 68.3 / 65.8, 4 of 32768 102.4 / 101.0, 2 of a ragged batch 102.4 /
+// 100.1 (8 tiles, one run: 66.4, 101.3, 101.8).
 constexpr int kItemTiles = 14;
 constexpr int kMidItemTiles = 12;                      // for a sequence
 constexpr int kMidFrom = 160, kMidTo = 512;            // of this many tiles
-constexpr int kFewRounds = 6, kMaxItemTiles = 16, kLseItemTiles = 4;
+constexpr int kFewRounds = 6, kMaxItemTiles = 16;
+constexpr int kLseFewRounds = 2, kLseItemTiles = 4;
 int long_item_tiles(int t) { return t >= kMidFrom && t <= kMidTo ? kMidItemTiles : kItemTiles; }
 int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int least, bool given_lse) {
     int active = 0;
@@ -604,12 +611,14 @@ int item_tiles(const std::vector<int>& tiles, int n_lb, int G, int least, bool g
         return (items * n_lb + G - 1) / G;
     };
     int best = 0, longest;
-    if (rounds(kItemTiles, &longest) > kFewRounds) return best;
-    if (given_lse) return std::max(least, kLseItemTiles);
+    const int64_t r14 = rounds(kItemTiles, &longest);
+    if (r14 > kFewRounds) return best;
+    if (given_lse && r14 > kLseFewRounds) return std::max(least, kLseItemTiles);
+    const float fixed = given_lse ? 1.f : 2.f, tail = given_lse ? 0.f : 0.25f;
     float best_cost = 0.f;
     for (int c = least; c <= kMaxItemTiles; ++c) {
         const float r = static_cast<float>(rounds(c, &longest));
-        const float cost = r * (static_cast<float>(longest) + 2.f) + 0.25f * static_cast<float>(longest);
+        const float cost = r * (static_cast<float>(longest) + fixed) + tail * static_cast<float>(longest);
         if (best_cost == 0.f || cost < best_cost) {
             best_cost = cost;
             best = c;

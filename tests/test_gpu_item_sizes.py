@@ -34,10 +34,11 @@ def test_item_lengths(case, max_ctas):
         gu.check_layer(wl, l, li, res[l], gu.run_oracle(wl, l, li, want_kv=False))
 
 
-# The given-lse kernel's items: of four tiles in a launch of up to six rounds (of 14-tile items), of 12 or
-# 14 tiles in one of more rounds or of more units than CTAs; a unit has at most as many items as CTAs.
+# The given-lse kernel's items: such that one or two rounds are full, of four tiles in a launch of up to six
+# rounds (of 14-tile items), of 12 or 14 tiles in one of more rounds or of more units than CTAs; a unit
+# has at most as many items as CTAs.
 # 8 units a layer on 8 CTAs: 84 tiles (10752 tokens) are six rounds, 85 are seven.
-LSE_CASES = [((129,), 1, 0), ((2433,), 2, 0), ((10752,), 1, 8), ((10753,), 1, 8), ((20480,), 1, 8), ((65537,), 1, 8),
+LSE_CASES = [((129,), 1, 0), ((16300,), 1, 0), ((20001, 900), 1, 0), ((2433,), 2, 0), ((10752,), 1, 8), ((10753,), 1, 8), ((20480,), 1, 8), ((65537,), 1, 8),
              ((8192, 100), 2, 0), ((900, 1, 3000), 1, 37), ((300,) * 20, 1, 0), ((2000,), 1, 1)]
 
 

@@ -45,3 +45,13 @@ def test_long_launches_cut_each_sequence_by_its_own_length(lse):
         if t >= 64:
             assert _items([t], 256, lse=lse) == [m]
     assert _items([161, 20000], 128, ctas=8, lse=lse) == [1, 8]
+
+
+@pytest.mark.parametrize("tiles,batches,want", [
+    ([16], 8, [16]), ([64], 8, [16]), ([128], 8, [19]), ([256], 8, [19]), ([32, 32], 16, [4, 4]),  # 1 or 2 rounds
+    ([64], 64, [16]), ([256], 32, [64]), ([256, 0, 3], 40, [64, 0, 1]),                            # 3 to 6
+    ([256], 56, [22]), ([300, 100], 100, [25, 8])])                                               # more, or many units
+def test_given_lse_items(tiles, batches, want):
+    """Full rounds of short items in a launch of one or two rounds, four tiles up to six rounds."""
+    ckv_build.build()
+    assert _items(tiles, batches, lse=True) == want

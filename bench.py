@@ -34,19 +34,20 @@ WORKLOAD = "needle_l131072"
 HBM_FALLBACK_GBS = 6800.0
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the scoring kernel per layer, per
-# workload, from an ncu capture of a two-layer launch of the same kernel (bench.py --layers 2 on
-# the workload), halved; keyed by the sha256 of the scoring kernels' sources (SCORE_SOURCES), so
-# a changed kernel reports null until it is captured again.  Rounded to 10 kB.  (Two layers of the
-# shorter workloads are a launch of few rounds, whose items are cut otherwise: none for their two-pass
-# scoring.)
+# workload, from an ncu capture of a launch over a few layers of the workload (bench.py --layers: 2 of
+# needle_l131072, 8 of llama8b_l32768, 5 of ragged_qwen7b: enough rounds that the items are cut as in the
+# whole model's launch), divided by them; keyed by the sha256 of the scoring kernels' sources
+# (SCORE_SOURCES), so a changed kernel reports null until it is captured again.  Rounded to 10 kB.
 SCORE_SOURCES = ('score_layers.cu', 'score_layers.cuh', 'score_resident.cu', 'score_lse.cu', 'score_common.cuh',
                  'ckv_device.cuh')
 SCORE_TRAFFIC = {
-    "2898cebd5566d56ca54ec15e05f1162e17c09172aa40873d287cdf34735dd502": {
-        "needle_l131072": 341_020_000,
-        "needle_l131072+lse": 272_180_000,
-        "llama8b_l32768+lse": 68_880_000,
-        "ragged_qwen7b+lse": 174_380_000,
+    "886e8257d83600ef251fbd54b1a3885da054b2a58149bd1ee4262b040bf9ba00": {
+        "needle_l131072": 339_180_000,
+        "llama8b_l32768": 71_890_000,
+        "ragged_qwen7b": 188_630_000,
+        "needle_l131072+lse": 272_140_000,
+        "llama8b_l32768+lse": 68_070_000,
+        "ragged_qwen7b+lse": 172_770_000,
     },
 }
 # Sequences up to this many tokens are selected by one block per (sequence, KV head)

@@ -80,10 +80,13 @@ typedef enum ckv_scope {
                               (the form Sec. 3.3 states); every KV head keeps those positions */
 } ckv_scope;
 
-/* Which scoring kernel runs the two passes over the keys (same scores either way). */
+/* Which scoring kernel runs the two passes over the keys (the same scores within the error bound).
+ * How a sequence's keys are split over CTAs, and with CKV_SCORE_AUTO which kernel runs, may depend on
+ * the call's other sequences and layers and on max_ctas: the same prompt's scores can differ in
+ * their last bits from call to call, and nearly equal candidates can then be chosen differently. */
 typedef enum ckv_score_path {
-    CKV_SCORE_AUTO = 0,     /* resident when it fits and N = 32 (see below) or the call is small,
-                               otherwise reload */
+    CKV_SCORE_AUTO = 0,     /* resident when it fits and N = 32 (see below) or the call is small
+                               (and of at most 65535 sequences), otherwise reload */
     CKV_SCORE_RESIDENT = 1, /* each key tile is read and multiplied once; pass 1 keeps its
                                exponentials in tensor memory and pass 2 rescales them.  Needs
                                every sequence's key tiles to fit one round of work items of at
@@ -352,8 +355,8 @@ CKV_API ckv_status ckv_allocate_budgets(const double* scores, int32_t num_layers
                                         int32_t max_budget, int32_t* budgets);
 
 /* Limit, for the calls enqueued after this one, of every bounded wait in which a kernel
- * waits on another of its roles or on another CTA: 0 restores the default (about 2 s).  When
- * a wait runs out the kernel sets CKV_DEV status 2 (a wait gave up) in the workspace status
+ * waits on another of its roles, on its loads or on another CTA: 0 restores the default (about
+ * 2 s).  When a wait runs out the kernel sets CKV_DEV status 2 (a wait gave up) in the workspace status
  * word, lets its own copies and MMAs finish, frees its tensor memory and returns; the results
  * of that call are then undefined, the CUDA context stays usable.  Process-wide; meant for
  * failure detection (and its tests), not for normal use. */

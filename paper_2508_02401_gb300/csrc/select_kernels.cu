@@ -471,8 +471,8 @@ __device__ __forceinline__ void pooled_values(const SelectParams& p, const UnitG
 
 // Copies the K and V rows of sequence-local positions list[0..m) to output rows
 // out_row0 + 0..m-1 of KV head g: a warp per row (16 lanes for K, 16 for V), kRowsInFlight
-// rows in flight per warp (not inlined: the rows in flight then stay in registers whatever the
-// caller holds).
+// rows in flight per warp (not inlined, so that the rows in flight do not compete with what the
+// caller holds; with the 64 registers of a 1024-thread block the loop spills 72 bytes all the same).
 constexpr int kRowsInFlight = 8;
 __device__ __noinline__ void copy_rows(const SelectParams& p, const UnitGeo& u, int kv,
                                           const int* list, int m, int out_row0) {
@@ -1272,11 +1272,13 @@ constexpr int kLsAhead = 2;     // score-row chunks asked into L2 ahead of the o
 constexpr int kLsCand = 2048;   // keys sharing the k-th key's first digit gathered in shared memory
 constexpr int kLsTies = 256;    // keys equal to the k-th key ranked by position in shared memory
 constexpr int kSelMaxLayers = 32;
-// kSelectOwnRows kept rows of a unit are copied by the CTA that selects them; the rest are cut into jobs of kLsJob rows
-// that the CTAs take once no unit is left, so that a large budget's rows (3072 of them took one SM
-// 80 us) spread over the GPU.  Selection and copies, us a call, own rows 256 / 512 / 1024 / all:
-// 32 layers at L = 32768, budgets up to 3072: 144 / 139 / 133 / 159; 8 ragged layers with the lse
-// given, budgets up to 1536, whole calls: 288 / 283 / 290 / 295 (with 512 threads and jobs of 256 rows).
+// kSelectOwnRows kept rows of a unit are copied by the CTA that selects them; the rest are cut into jobs of
+// kLsJob rows that the CTAs take once no unit is left, so that a large budget's rows (17 ns each on one
+// SM) spread over the GPU.  Calls with the lse given, us, jobs beyond 1024 rows / no jobs: 32 layers of 32768
+// tokens, mean budget 1024 461 / 462, 1400 482 / 490; 16 of 16384, 2048 207 / 217; 8 of 131072, 2048 586 /
+// 610; where every SM has rows of its own they cost: 28 ragged layers, 2048 1184 / 1144, 2 of 32768, 2048
+// 131 / 125.  Own rows 256 / 512 / 1024 / 2048: 32 of 32768 468 / 466 / 461 / 463, 8 ragged 278 / 279 / 284 /
+// 285.  Jobs of 256 / 512 / 1024 rows: 462 / 461 / 464, 2 of 32768 131 / 130 / 123.
 constexpr int kLsJob = 512;
 
 struct SelectLayersParams {
